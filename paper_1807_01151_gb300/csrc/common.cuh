@@ -65,11 +65,13 @@ struct Lv {
 struct LevelDev {
     int p = 0, N = 0, q = 0, Q = 0, QF = 0, B = 0;
     // quadrature tables (per element / per face)
-    double* vpsi = nullptr;    // [E][Q][N]      psi_i(x_q)
-    double* vgw = nullptr;     // [E][D][Q][N]   W_q d_k psi_i(x_q)
+    // (p >= 1: fixed point, fix.cuh, two 32-bit halves in the place of each float64; p = 0: float64)
+    double* vpsi = nullptr;    // [E][N][Q]      psi_i(x_q)
+    double* vgw = nullptr;     // [E][D][Q][N]   W_q d_k psi_i(x_q)  (fixed point: rows q D + k, GradTab)
+    int2* texp = nullptr;      // [E]            their exponents: of psi (volume and face points), of vgw
     double* fnrm = nullptr;    // [F][QF][3]     unit outward normal of the L element
     double* famag = nullptr;   // [F][QF]        w |n dS|
-    double* fpsiL = nullptr;   // [F][QF][N]     psi^L_i at the face points
+    double* fpsiL = nullptr;   // [F][QF][N]     psi^L_i at the face points  (fixed point: FaceTab)
     double* fpsiR = nullptr;   // [F_int][QF][N] psi^R_i at the face points
     double* fwn = nullptr;     // [F-F_int][QF][3] slip-wall reflection normal (body normal)
     double* vvr = nullptr;     // [E][Q][3]      frame velocity omega x x (rotating frame only)
@@ -81,7 +83,11 @@ struct LevelDev {
     double* un = nullptr;      // u^n of the PRK step
     double* r = nullptr;       // residual work
     double* r2 = nullptr;      // second residual buffer
-    double* fhat = nullptr;    // [F][QF][5]     w|n dS| F~ at the face points
+    double* tr = nullptr;      // [F][QF][2][5]  U_h on the two sides of the face points (p >= 1)
+    double* trj = nullptr;     // the same for the FP64 face Jacobians (FP64 form: a buffer of its own,
+                               // the side stream may be evaluating residuals; else tr)
+    double* fhat = nullptr;    // [F][QF][5]     w|n dS| F~ at the face points (p >= 1: fixed point, [F][QF][6])
+    int* fkey = nullptr;       // [F][5]         largest key of a face's fluxes (p >= 1)
     double* fjl = nullptr;     // [F][QF][25]    w|n dS| dF~/dU_L (boundary: total derivative)
     double* fjr = nullptr;     // [F_int][QF][25] w|n dS| dF~/dU_R
     double* blk = nullptr;     // [E][B][B]      P_e, then its LU factors (column-major)
@@ -243,6 +249,8 @@ struct ProfScope {
 namespace emg {
 emg_status setup_device_mesh(emg_ctx* c, const emg_mesh_desc* m);
 emg_status launch_residual(emg_ctx* c, int p, const double* u, const double* tau, double* R);
+emg_status launch_traces(emg_ctx* c, int p, const double* u, double* tr, int cls);
+emg_status fix_tables(emg_ctx* c);
 emg_status launch_face_jacobian(emg_ctx* c, int p, const double* u);
 emg_status launch_diag_blocks(emg_ctx* c, int p, const double* u, const double* cfl_dev, int shifted,
                               double* out);

@@ -1,0 +1,125 @@
+// Float64 dot products on the integer pipe.  GB300 issues 2 float64 multiply-adds per clock and
+// SM, but more than 40 32 x 32 -> 64 bit integer ones, so the residual's contractions (traces,
+// volume quadrature, projections) take their factors as fixed-point numbers of 56 bits and sign:
+//   x = v 2^-s,  v = hi 2^28 + lo,  |v| < 2^56,  -2^27 <= lo < 2^27,
+// one exponent s for each group of factors that is summed over (an element's basis table, an
+// element's coefficients or fluxes of one variable), taken from the group's largest magnitude.
+// Three multiply-adds per term keep the exact sums
+//   h = sum hi hi',  x = sum (hi lo' + lo hi')
+// and the result is (h 2^56 + x 2^28) 2^(-s-s'); the terms lo lo' (below 2^-58 of the largest
+// term) are left out.  With at most FIX_TERMS = 120 terms neither sum can overflow:
+// |h|, |x| <= 120 2^56 < 2^63.  Against float64 multiply-adds, which round at 2^-53 of the running
+// sum at every term, the factors are cut at 2^-56 of their group's largest, once.  Measured
+// against 64-bit references both forms' errors are the same (rounding of the result).
+// A group that holds an infinity or a NaN gets the scale NaN, so every sum over it is NaN.
+#pragma once
+
+#include "common.cuh"
+
+namespace emg {
+
+constexpr int FIX_LO = 28;      // bits of the low half
+constexpr int FIX_BITS = 56;    // |v| < 2^FIX_BITS
+constexpr int FIX_TERMS = 120;  // most terms of one sum
+
+// Magnitude key of x: its high word without the sign (orders like |x| up to the low word).
+__device__ __forceinline__ int fix_key(double x) { return __double2hiint(x) & 0x7fffffff; }
+
+// Exponent s of a group whose largest key is `key`: |x| 2^s < 2^56 for every member.  Groups below
+// 2^-900 share the exponent of 2^-900 (their members become small integers or 0).
+__device__ __forceinline__ int fix_exp(int key) {
+    const int f = key >> 20;
+    return FIX_BITS + 1022 - (f < 123 ? 123 : f);
+}
+
+// 2^e as a double, NaN where the group's key is not that of a finite number.
+__device__ __forceinline__ double fix_scale(int e, int key) {
+    const int b = 1023 + e;
+    const double s = b >= 2047 ? __hiloint2double(0x7ff00000, 0) : b <= 0 ? 0.0 : __hiloint2double(b << 20, 0);
+    return key >= 0x7ff00000 ? __hiloint2double(0x7ff80000, 0) : s;
+}
+
+// v = x 2^s cut to an integer, as (hi, lo); |x| 2^s < 2^56.
+__device__ __forceinline__ int2 fix_of(double x, int s) {
+    const int hw = __double2hiint(x);
+    const int sh = 1078 - s - ((hw >> 20) & 0x7ff);   // |v| = (mantissa 2^3) >> sh, sh >= 0
+    const unsigned long long m =
+        (((unsigned long long)((hw & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x)) << 3;
+    const unsigned long long a = sh > 63 ? 0ull : m >> sh;
+    const long long v = hw < 0 ? -(long long)a : (long long)a;
+    return make_int2((int)((v + (1ll << (FIX_LO - 1))) >> FIX_LO), ((int)v << (32 - FIX_LO)) >> (32 - FIX_LO));
+}
+
+// (hi, lo) of v 2^-k, k >= 0, negated where neg is set.
+__device__ __forceinline__ int2 fix_shift(int2 p, int k, bool neg) {
+    long long v = ((long long)p.x << FIX_LO) + (long long)p.y;
+    v >>= k > 63 ? 63 : k;
+    if (neg) v = -v;
+    return make_int2((int)((v + (1ll << (FIX_LO - 1))) >> FIX_LO), ((int)v << (32 - FIX_LO)) >> (32 - FIX_LO));
+}
+
+// v as a double (v 2^-s is the number it stands for).
+__device__ __forceinline__ double fix_back(int2 v) {
+    return __ll2double_rn(((long long)v.x << FIX_LO) + (long long)v.y);
+}
+
+__device__ __forceinline__ void fix_mac(long long& h, long long& x, int2 a, int2 b) {
+    h += (long long)a.x * b.x;
+    x += (long long)a.x * b.y;
+    x += (long long)a.y * b.x;
+}
+
+// The sum as a double; scale = 2^(56 - s - s').
+__device__ __forceinline__ double fix_sum(long long h, long long x, double scale) {
+    return __ll2double_rn(h + ((x + (1ll << (FIX_LO - 1))) >> FIX_LO)) * scale;
+}
+
+// Layout of the projections' tables: rows (points) of N modes, two consecutive rows interleaved,
+// [R / 2][N][2] (an odd last row follows alone), so that a thread, which owns a mode, takes two rows
+// with one 16-byte load.  Face tables whose sides would not start on 16 bytes stay [QF][N].
+template <int N, int ROWS, bool PAIRED>
+struct RowTab {
+    static constexpr bool paired = PAIRED;
+    __host__ __device__ static constexpr int at(int r, int i) {
+        return !PAIRED || r >= (ROWS & ~1) ? r * N + i : ((r >> 1) * N + i) * 2 + (r & 1);
+    }
+    __host__ __device__ static constexpr int row(int o) {
+        return !PAIRED || o >= (ROWS & ~1) * N ? o / N : o / (2 * N) * 2 + (o & 1);
+    }
+    __host__ __device__ static constexpr int mode(int o) {
+        return !PAIRED || o >= (ROWS & ~1) * N ? o % N : (o % (2 * N)) >> 1;
+    }
+};
+template <int D, int P>
+using FaceTab = RowTab<Lv<D, P>::N, Lv<D, P>::QF, (Lv<D, P>::QF * Lv<D, P>::N) % 2 == 0>;
+// weighted gradients: row q D + k of element e
+template <int D, int P>
+using GradTab = RowTab<Lv<D, P>::N, D * Lv<D, P>::Q, (D * Lv<D, P>::Q * Lv<D, P>::N) % 2 == 0>;
+
+// Ask L2 for `bytes` bytes from p (any alignment): one instruction, no register, nothing waits.
+__device__ __forceinline__ void l2_prefetch(const void* p, size_t bytes) {
+    const uint64_t a = reinterpret_cast<uint64_t>(p) & ~(uint64_t)15;
+    const unsigned n = (unsigned)((reinterpret_cast<uint64_t>(p) + bytes + 15 - a) & ~(uint64_t)15);
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(reinterpret_cast<void*>(a))), "r"(n)
+                 : "memory");
+}
+
+// Reciprocal and reciprocal square root of a float64: one third-order step (Householder's method
+// for 1/y - a and 1/y^2 - a) on the hardware's approximation, whose error of about 2^-20 becomes
+// its cube, below the rounding of the result (within 2 ulp of the exact value).  3 and 5 float64
+// operations, where the correctly rounded division and square root take the pipe for 5 and 9.  For
+// normal positive arguments; 0, denormals and infinities give an infinity or NaN.
+__device__ __forceinline__ double rcp_h3(double a) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt_h3(double a) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a * y, y, 1.0);
+    return fma(e * y, fma(0.375, e, 0.5), y);
+}
+
+}  // namespace emg

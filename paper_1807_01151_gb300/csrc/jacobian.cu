@@ -17,6 +17,7 @@
 #include "common.cuh"
 #include "dispatch.cuh"
 #include "euler.cuh"
+#include "fix.cuh"
 #include "jacobian.cuh"
 
 namespace emg {
@@ -81,10 +82,11 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
     const int* __restrict__ elem_face, const T* __restrict__ fpsiL, const T* __restrict__ fpsiR,
     const T* __restrict__ fjl, const T* __restrict__ fjr, const double* __restrict__ psic,
     const double* __restrict__ hlen, const double* __restrict__ cfl_dev, double g, int shifted,
-    const double* __restrict__ vvr, T* __restrict__ out) {
+    const double* __restrict__ vvr, const int2* __restrict__ texp, T* __restrict__ out) {
     using L = Lv<D, P>;
     constexpr int N = L::N, Q = L::Q, QF = L::QF, B = L::B, NF = L::NF;
     constexpr int QC = DiagCfg<D, P>::QC;
+    constexpr bool FX = P > 0 && sizeof(T) == 8;   // the float64 tables of p >= 1 are fixed point
     constexpr int VL = Vec16<T>::L, NP = ((N + VL - 1) / VL) * VL;   // padded basis rows
     // the finished block goes out through shared memory (coalesced) when it fits
     constexpr bool STAGE = (size_t)B * B * sizeof(T) <= 24576;
@@ -120,6 +122,11 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
         const double cs = sqrt(g * pr * ir);
         s_dtau = cfl_dev[0] * hlen[e] / ((2 * P + 1) * (sqrt(q2) + cs));
     }
+    double s_psi = 1.0, s_gw = 1.0;
+    if constexpr (FX) {
+        const int2 te = texp[e];
+        s_psi = fix_scale(-te.x, 0), s_gw = fix_scale(-te.y, 0);
+    }
     const bool active = tid < 25 * N;
     const int ab = tid / N, i = tid % N;
     const int a = ab / 5, b = ab % 5;
@@ -132,17 +139,30 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
             __syncthreads();
             // stage the chunk's psi and W grad psi, and build U at its points (all threads)
             const T* pg = vpsi + ((size_t)e * Q + q0) * N;
-            for (int t = tid; t < nq * NP; t += blockDim.x) {
-                const int q = t / NP, j = t % NP;
-                ps[q][j] = j < N ? pg[q * N + j] : (T)0;
+            if constexpr (FX) {   // stored [N][Q]
+                const int2* pf = reinterpret_cast<const int2*>(vpsi) + (size_t)e * Q * N + q0;
+                for (int t = tid; t < nq * NP; t += blockDim.x) {
+                    const int j = t / nq, q = t % nq;
+                    ps[q][j] = j < N ? fix_back(pf[j * Q + q]) * s_psi : 0.0;
+                }
+                __syncthreads();
+            } else {
+                for (int t = tid; t < nq * NP; t += blockDim.x) {
+                    const int q = t / NP, j = t % NP;
+                    ps[q][j] = j < N ? pg[q * N + j] : (T)0;
+                }
             }
             for (int t = tid; t < D * nq * N; t += blockDim.x) {
                 const int k = t / (nq * N), r = t % (nq * N);
-                gs[r / N][k][r % N] = vgw[(((size_t)e * D + k) * Q + q0) * N + r];
+                if constexpr (FX)
+                    gs[r / N][k][r % N] = fix_back(reinterpret_cast<const int2*>(
+                        vgw)[(size_t)e * D * Q * N + GradTab<D, P>::at((q0 + r / N) * D + k, r % N)]) * s_gw;
+                else
+                    gs[r / N][k][r % N] = vgw[(((size_t)e * D + k) * Q + q0) * N + r];
             }
             for (int t = tid; t < nq * 5; t += blockDim.x) {
                 const int q = t / 5, c = t % 5;
-                const T* pq = pg + (size_t)q * N;
+                const T* pq = FX ? ps[q] : pg + (size_t)q * N;
                 T s = (T)0;
                 for (int m = 0; m < N; ++m) s += us[c * N + m] * pq[m];
                 Us[q][c] = s;
@@ -177,7 +197,10 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
         __syncthreads();
         for (int t = tid; t < QF * NP; t += blockDim.x) {
             const int q = t / NP, j = t % NP;
-            fps[q][j] = j < N ? pt[q * N + j] : (T)0;
+            if constexpr (FX)
+                fps[q][j] = j < N ? fix_back(reinterpret_cast<const int2*>(pt)[FaceTab<D, P>::at(q, j)]) * s_psi : 0.0;
+            else
+                fps[q][j] = j < N ? pt[q * N + j] : (T)0;
         }
         for (int t = tid; t < QF * 25; t += blockDim.x) fjs[t / 25][t % 25] = (code & 1) ? fj[t] : -fj[t];
         __syncthreads();
@@ -529,7 +552,7 @@ emg_status launch_diag_blocks(emg_ctx* c, int p, const double* u, const double* 
         ProfScope _ps(c, PC_DIAG);                                                                          \
         k_diag_blocks<DD, PP, double><<<(unsigned)c->E, DiagCfg<DD, PP>::THREADS, 0, c->stream>>>(          \
             (int)c->E, nmax, u, L.vpsi, L.vgw, c->elem_face, L.fpsiL, L.fpsiR, L.fjl, L.fjr, c->psic, c->h, \
-            cfl_dev, c->prm.gamma, shifted, L.vvr, out);                                                    \
+            cfl_dev, c->prm.gamma, shifted, L.vvr, L.texp, out);                                            \
     }
     EMG_DISPATCH_DP(c->dim, p, EMG_DB)
 #undef EMG_DB
@@ -557,7 +580,7 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
         if (c->prm.block_kernels == 3)                                                                      \
             k_diag_blocks<DD, PP, float><<<(unsigned)c->E, DiagCfg<DD, PP>::THREADS, 0, c->stream>>>(       \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
-                c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, out);                                 \
+                c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, nullptr, out);                        \
         else                                                                                                \
             k_diag_blocks_rb<DD, PP><<<(unsigned)c->E, DiagRb<DD, PP>::THREADS, 0, c->stream>>>(            \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \

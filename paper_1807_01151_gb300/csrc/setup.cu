@@ -429,6 +429,8 @@ int64_t estimate_bytes(int dim, int64_t E, int64_t F, int64_t F_int, int p_max, 
         b += 6 * E * B * 8;                                                     // v, v0, tau, un, r, r2
         if (rot) b += (E * Q + F * QF) * 3 * 8;                                 // frame velocities
         if (p > 0) {
+            b += E * 8 + F * (QF * 8 + 5 * 4);                                   // table exponents, fluxes
+            b += F * QF * 10 * 8 * (blocks_f32(prec) ? 1 : 2);                   // traces
             if (blocks_f32(prec))
                 b += E * B * B * 4 + E * Q * N * (1 + dim) * 4 + F * QF * (N + 25) * 4 + Fi1 * QF * (N + 25) * 4;
             else
@@ -598,7 +600,14 @@ emg_status setup_device_mesh(emg_ctx* c, const emg_mesh_desc* m) {
         EMG_ALLOC(L.un, double, S);
         EMG_ALLOC(L.r, double, S);
         EMG_ALLOC(L.r2, double, S);
-        EMG_ALLOC(L.fhat, double, F * L.QF * 5);
+        EMG_ALLOC(L.fhat, double, F * L.QF * (p > 0 ? 6 : 5));
+        if (p > 0) {
+            EMG_ALLOC(L.fkey, int, F * 5);
+            EMG_ALLOC(L.texp, int2, E);
+            EMG_ALLOC(L.tr, double, F * L.QF * 10);
+            L.trj = L.tr;
+            if (!blocks_f32(c->prm.prec)) EMG_ALLOC(L.trj, double, F * L.QF * 10);
+        }
         EMG_ALLOC(L.fjl, double, F * L.QF * 25);
         EMG_ALLOC(L.fjr, double, std::max<int64_t>(F_int, 1) * L.QF * 25);
         if (c->rot) {
@@ -683,6 +692,8 @@ emg_status setup_device_mesh(emg_ctx* c, const emg_mesh_desc* m) {
         st = tune_gj(c);
         if (st != EMG_OK) return st;
     }
+    st = fix_tables(c);
+    if (st != EMG_OK) return st;
     std::vector<double> hv(E);
     EMG_CUDA_TRY(c, cudaMemcpyAsync(hv.data(), c->vol, E * 8, cudaMemcpyDeviceToHost, c->stream));
     EMG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
