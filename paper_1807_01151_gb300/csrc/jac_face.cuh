@@ -1,8 +1,8 @@
 // Face Jacobians of the exact Jacobian blocks (Sec. 3.3): k_face_jac, per face point,
 // dF~/dU_L and dF~/dU_R of the Roe flux by forward-mode AD (Dual<5>); on boundary faces the
 // total derivative through the ghost state, dF~/dU_L + dF~/dU_ghost dU_ghost/dU_L;
-// k_face_jac_col the same, one derivative direction per thread.  Instantiated for FP64 in
-// jac_face.cu and for float32 in jac_face32.cu (2-D) and jac_face32_3d.cu (3-D).
+// k_face_jac_col the same, one derivative direction per thread.  Instantiated for float32 in
+// jac_face32.cu (2-D) and jac_face32_3d.cu (3-D); the FP64 ones are in jac_face.cu.
 #pragma once
 
 #include "common.cuh"
@@ -53,21 +53,18 @@ __global__ void __launch_bounds__(128) k_face_jac(int F, int F_int, const int* _
                                                   const S* __restrict__ fpsiL,
                                                   const S* __restrict__ fpsiR,
                                                   const double* __restrict__ fwn,
-                                                  const double* __restrict__ u, const double* __restrict__ tr,
-                                                  double g, U5 uinf, const double* __restrict__ fvr,
+                                                  const double* __restrict__ u, double g, U5 uinf,
+                                                  const double* __restrict__ fvr,
                                                   S* __restrict__ fjl, S* __restrict__ fjr) {
     using L = Lv<D, P>;
     constexpr int N = L::N, QF = L::QF;
-    constexpr bool TR = P > 0 && sizeof(S) == 8;   // traces from k_traces (the FP64 tables are fixed point)
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)F * QF) return;
     const int f = (int)(idx / QF);
     const double n[3] = {fnrm[idx * 3], fnrm[idx * 3 + 1], fnrm[idx * 3 + 2]};
     const S am = (S)famag[idx];
     S UL[5];
-    if constexpr (TR) {
-        for (int a = 0; a < 5; ++a) UL[a] = tr[idx * 10 + a];
-    } else {
+    {
         const double* ue = u + (size_t)fL[f] * 5 * N;
         const S* ps = fpsiL + idx * N;
         for (int a = 0; a < 5; ++a) {
@@ -82,15 +79,11 @@ __global__ void __launch_bounds__(128) k_face_jac(int F, int F_int, const int* _
         dL[a].d[a] = (S)1;
     }
     if (f < F_int) {
+        const double* ur = u + (size_t)fR[f] * 5 * N;
+        const S* pr = fpsiR + idx * N;
         for (int a = 0; a < 5; ++a) {
             S s = (S)0;
-            if constexpr (TR) {
-                s = tr[idx * 10 + 5 + a];
-            } else {
-                const double* ur = u + (size_t)fR[f] * 5 * N;
-                const S* pr = fpsiR + idx * N;
-                for (int i = 0; i < N; ++i) s += (S)ur[a * N + i] * pr[i];
-            }
+            for (int i = 0; i < N; ++i) s += (S)ur[a * N + i] * pr[i];
             dR[a] = dconst<5, S>(s);
         }
         face_flux_d<ROT>(dL, dR, n, g, fvr, idx, Fd);
@@ -193,11 +186,11 @@ void face_jacobian32_go(emg_ctx* c, const double* u) {
     if (c->prm.block_kernels == 3 && c->rot)
         k_face_jac<D, P, float, true><<<g1, 128, 0, c->stream>>>(
             F, Fi, c->face_L, c->face_R, c->face_bc, L.fnrm, L.famag, L.fpsiL32, L.fpsiR32, L.fwn, u,
-            nullptr, c->prm.gamma, ui, L.fvr, L.fjl32, L.fjr32);
+            c->prm.gamma, ui, L.fvr, L.fjl32, L.fjr32);
     else if (c->prm.block_kernels == 3)
         k_face_jac<D, P, float, false><<<g1, 128, 0, c->stream>>>(
             F, Fi, c->face_L, c->face_R, c->face_bc, L.fnrm, L.famag, L.fpsiL32, L.fpsiR32, L.fwn, u,
-            nullptr, c->prm.gamma, ui, nullptr, L.fjl32, L.fjr32);
+            c->prm.gamma, ui, nullptr, L.fjl32, L.fjr32);
     else if (c->rot)
         k_face_jac_col<D, P, float, true><<<gc, 128, 0, c->stream>>>(
             F, Fi, c->face_L, c->face_R, c->face_bc, L.fnrm, L.famag, L.fpsiL32, L.fpsiR32, L.fwn, u,
