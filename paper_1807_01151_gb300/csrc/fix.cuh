@@ -63,10 +63,15 @@ __device__ __forceinline__ double fix_back(int2 v) {
     return __ll2double_rn(((long long)v.x << FIX_LO) + (long long)v.y);
 }
 
+// In PTX: from the C++ form the compiler makes 64 x 64 bit products where a factor was split from a
+// 64-bit value in registers (measured: 6 instructions in place of each).
+__device__ __forceinline__ void fix_mad(long long& h, int a, int b) {
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(h) : "r"(a), "r"(b));
+}
 __device__ __forceinline__ void fix_mac(long long& h, long long& x, int2 a, int2 b) {
-    h += (long long)a.x * b.x;
-    x += (long long)a.x * b.y;
-    x += (long long)a.y * b.x;
+    fix_mad(h, a.x, b.x);
+    fix_mad(x, a.x, b.y);
+    fix_mad(x, a.y, b.x);
 }
 
 // The sum as a double; scale = 2^(56 - s - s').

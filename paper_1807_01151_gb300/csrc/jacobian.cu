@@ -545,10 +545,15 @@ static emg_status add_source_jacobian(emg_ctx* c, int p, int shifted, T* out) {
 emg_status launch_diag_blocks(emg_ctx* c, int p, const double* u, const double* cfl_dev, int shifted, double* out) {
     emg_status st = launch_face_jacobian(c, p, u);
     if (st != EMG_OK) return st;
+    if (diag_blocks_fx_serves(c->dim, p)) {
+        st = launch_diag_blocks_fx(c, p, u, cfl_dev, shifted, out);
+        if (st != EMG_OK) return st;
+        return add_source_jacobian(c, p, shifted, out);
+    }
     LevelDev& L = c->lv[p];
     const int nmax = n_modes(c->dim, c->p_max);
 #define EMG_DB(DD, PP)                                                                                      \
-    {                                                                                                       \
+    if constexpr (PP == 0 || (DD == 3 && PP == 4)) {                                                        \
         ProfScope _ps(c, PC_DIAG);                                                                          \
         k_diag_blocks<DD, PP, double><<<(unsigned)c->E, DiagCfg<DD, PP>::THREADS, 0, c->stream>>>(          \
             (int)c->E, nmax, u, L.vpsi, L.vgw, c->elem_face, L.fpsiL, L.fpsiR, L.fjl, L.fjr, c->psic, c->h, \

@@ -1,6 +1,7 @@
 // Pieces of the exact Jacobian blocks (Sec. 3.3) shared by the translation units that build
-// them: jacobian.cu (SIMT assembly, p = 0 blocks, source term, launchers), jac_face.cu (face
-// Jacobians by dual numbers) and jac_tc.cu (tensor-core assembly of the float32 forms).
+// them: jacobian.cu (SIMT assembly, p = 0 blocks, source term, launchers), jac_face*.cu (face
+// Jacobians), jac_fix.cu (FP64 assembly in fixed point) and jac_tc.cu (tensor-core assembly of the
+// float32 forms).
 #pragma once
 
 #include "common.cuh"
@@ -68,5 +69,10 @@ emg_status launch_face_jacobian32(emg_ctx* c, int p, const double* u);
 // without the rotating frame's source term, which the caller adds.
 emg_status launch_diag_blocks_tc(emg_ctx* c, int p, const double* u, const double* cfl_dev, int shifted,
                                  float* out);
+
+// FP64 assembly on the integer pipe (jac_fix.cu): which levels it serves, and its launch (P_e or
+// D_e without the rotating frame's source term).
+bool diag_blocks_fx_serves(int dim, int p);
+emg_status launch_diag_blocks_fx(emg_ctx* c, int p, const double* u, const double* cfl_dev, int shifted, double* out);
 
 }  // namespace emg

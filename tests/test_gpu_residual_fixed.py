@@ -1,4 +1,4 @@
-"""The residual's fixed-point contractions (traces, volume quadrature, projections) against the
+"""The residual's and the FP64 blocks' fixed-point contractions (traces, volume quadrature, projections) against the
 oracle: element counts that leave the last block short, both splits of the projection (few
 elements: four threads per mode), every order, a spanwise momentum in 2-D, and non-finite input.
 
@@ -65,3 +65,23 @@ def test_non_finite_coefficient_stays_with_its_neighbours(size, bad):
     touched[[e] + list(dg.mesh.neighbours[e])] = True
     assert not np.isfinite(R[touched]).all(axis=(1, 2)).any()
     assert np.array_equal(R[~touched], clean[~touched])
+
+
+@pytest.mark.parametrize("dim,size,p", [(2, (7, 3), 0), (2, (7, 3), 1), (2, (7, 3), 2), (2, (5, 3), 3), (2, (5, 2), 4),
+                                        (3, (1, 2), 1), (3, (1, 2), 2), (3, (1, 1), 3)])
+def test_diagonal_blocks_match_oracle(dim, size, p):
+    """Blocks (face Jacobians and assembly) with and without a spanwise momentum in 2-D; the bound is
+    that of the other FP64 block tests."""
+    desc = ogrid(*size) if dim == 2 else cubed_sphere_shell(*size)
+    dg = DG(desc, p)
+    u = perturbed_state(dg, seed=21 + p)
+    s = _solver(desc, p)
+    for spanwise in ([False, True] if dim == 2 else [True]):
+        if dim == 2 and spanwise:
+            u[::3, 3, :] = 0.05 * u[::3, 1, :]
+        D = s.jacobian_diag(p, u)
+        Do = dg.diag_blocks(p, u)
+        assert np.abs(D - Do).max() <= 1e-11 * np.abs(Do).max()
+        for e in range(dg.E):   # element by element too: their scales differ by the mesh's stretching
+            assert np.abs(D[e] - Do[e]).max() <= 1e-11 * np.abs(Do[e]).max()
+    s.close()
