@@ -1,4 +1,4 @@
-"""The residual's and the FP64 blocks' fixed-point contractions (traces, volume quadrature, projections) against the
+"""The residual's and the FP64 blocks' fixed-point contractions (and the blocks' factorisation) (traces, volume quadrature, projections) against the
 oracle: element counts that leave the last block short, both splits of the projection (few
 elements: four threads per mode), every order, a spanwise momentum in 2-D, and non-finite input.
 
@@ -85,3 +85,29 @@ def test_diagonal_blocks_match_oracle(dim, size, p):
         for e in range(dg.E):   # element by element too: their scales differ by the mesh's stretching
             assert np.abs(D[e] - Do[e]).max() <= 1e-11 * np.abs(Do[e]).max()
     s.close()
+
+
+@pytest.mark.parametrize("size,p", [((7, 3), 1), ((7, 3), 2), ((5, 3), 3), ((5, 2), 4)])
+@pytest.mark.parametrize("state,forcing", [(False, False), (True, False), (False, True)])
+def test_fp64_prk_step_with_and_without_spanwise_momentum(size, p, state, forcing):
+    """The FP64 factorisation splits blocks whose spanwise momentum is uncoupled: plane flow (split,
+    spanwise part of the residual 0), plane flow with a spanwise forcing (split, both systems solved)
+    and a state with a spanwise momentum (whole blocks).  The bound is that of the FP64 PRK tests."""
+    from oracle import emg as oemg
+    desc = ogrid(*size)
+    dg = DG(desc, p)
+    u = perturbed_state(dg, seed=31 + p)
+    tau = np.zeros_like(u)
+    if state:
+        u[::3, 3, :] = 0.05 * u[::3, 1, :]
+    if forcing:
+        tau[:, 3, :] = 1e-3 * u[:, 0, :]
+    s = _solver(desc, p)
+    out = s.prk_step(p, u, tau=tau, cfl=5.0)
+    s.close()
+    D = dg.diag_blocks(p, u)
+    P = np.eye(D.shape[-1])[None] / oemg.dtau(dg, p, u, 5.0)[:, None, None] - D
+    ref = oemg.prk_step(lambda w: dg.residual(p, w) + tau, P, u)
+    assert np.abs(out - ref).max() <= 1e-11 * np.abs(ref).max()
+    if not (state or forcing):
+        assert not out[:, 3].any()
