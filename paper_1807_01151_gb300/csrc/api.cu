@@ -7,6 +7,7 @@
 #include <new>
 #include <vector>
 
+#include "blocks.cuh"
 #include "common.cuh"
 
 using namespace emg;
@@ -70,15 +71,28 @@ __global__ void k_set_freestream(int64_t E, int N, const double* __restrict__ vo
     v[idx] = i == 0 ? U[a] * sqrt(vol[e]) : 0.0;
 }
 
-// float32 blocks widened to float64 row-major (colmajor: the source is column-major)
+// float32 blocks widened to float64 row-major (colmajor: the source is column-major; split: flags of
+// the elements that are packed, blocks.cuh, or null)
 __global__ void k_widen_blocks(int64_t E, int B, const float* __restrict__ src, int colmajor,
-                               double* __restrict__ dst) {
+                               const int* __restrict__ split, double* __restrict__ dst) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t BB = (int64_t)B * B;
     if (t >= E * BB) return;
     const int64_t e = t / BB;
     const int rc = (int)(t % BB);
     const int r = rc / B, cc = rc % B;
+    if (split && split[e]) {
+        const int N = B / 5, rs = r / N, cs = cc / N, B4 = 4 * N;
+        const float* p = src + gj_packed_at(e, B);
+        float v = 0.0f;
+        if (rs != 3 && cs != 3)
+            v = colmajor ? p[(cs == 4 ? cc - N : cc) * B4 + (rs == 4 ? r - N : r)]
+                         : p[(rs == 4 ? r - N : r) * B4 + (cs == 4 ? cc - N : cc)];
+        else if (rs == cs)
+            v = p[B4 * B4 + (colmajor ? (cc - 3 * N) * N + r - 3 * N : (r - 3 * N) * N + cc - 3 * N)];
+        dst[t] = (double)v;
+        return;
+    }
     dst[t] = (double)src[e * BB + (colmajor ? (int64_t)cc * B + r : (int64_t)r * B + cc)];
 }
 
@@ -697,7 +711,9 @@ emg_status emg_block_operator(emg_ctx* c, int32_t p, const double* u, double cfl
         }
         const int64_t tot = n * B;
         { ProfScope _ps(c, PC_CONTROL); k_widen_blocks<<<(unsigned)((tot + 255) / 256), 256, 0, c->stream>>>(
-            c->E, B, L.blk32, which, Dd); }
+            c->E, B, L.blk32, which, 
+            which == 1 ? (L.gj_split ? gj_work(L.piv, c->E).flag : nullptr) : L.asm_plane ? gj_work(L.piv, c->E).asm_flag : nullptr,
+            Dd); }
         EMG_CHECK_LAUNCH(c);
     } else {
         st = launch_diag_blocks(c, p, L.un, &c->sc->cfl, 1, L.blk);

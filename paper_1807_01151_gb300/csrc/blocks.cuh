@@ -29,6 +29,34 @@ __device__ __forceinline__ void fma2f(float a, float b0, float b1, float& d0, fl
     d1 = r.y;
 }
 
+// Where the packed form of element e starts (floats, 16-byte aligned, within the element's B x B
+// place), for blocks that split only (gj.cu): the 4 N x 4 N system over variables 0, 1, 2, 4, then the
+// N x N one of variable 3, row-major from the assembly (jac_plane.cu), column-major once inverted.
+__host__ __device__ __forceinline__ size_t gj_packed_at(int64_t e, int B) { return ((size_t)e * B * B + 3) & ~(size_t)3; }
+
+// Work space of the split float32 blocks of a 2-D level, in the E x B integers of LevelDev::piv (B >=
+// 15): flags of the packed blocks and list of the others, of the assembly and of the inverse.  head: the
+// list's length and a ticket.
+struct GjWork {
+    int *flag, *list, *head, *asm_flag, *asm_list, *asm_head;
+};
+inline GjWork gj_work(int* w, int64_t E) { return {w, w + E, w + 4 * E, w + 2 * E, w + 3 * E, w + 4 * E + 2}; }
+
+// Length of a list, read by every CTA of a grid; the last one out sets it back to 0.
+__device__ __forceinline__ int take_list(int* head) {
+    const int n = *reinterpret_cast<volatile int*>(head);
+    __syncthreads();   // every thread has read it
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(head + 1, 1) == (int)gridDim.x - 1) {   // every CTA has
+            head[0] = 0;
+            head[1] = 0;
+        }
+    }
+    return n;
+}
+constexpr unsigned kListBlocks = 608;   // CTAs that share a list: four per SM
+
 // B = 5 N(p): 2-D p = 1..4, then 3-D p = 1..4 (B = 50 serves both dimensions).
 #define EMG_BSIZES(X) X(15) X(30) X(50) X(75) X(20) X(100) X(175)
 

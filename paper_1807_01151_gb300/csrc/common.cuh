@@ -91,7 +91,7 @@ struct LevelDev {
     double* fjl = nullptr;     // [F][QF][25]    w|n dS| dF~/dU_L (boundary: total derivative)
     double* fjr = nullptr;     // [F_int][QF][25] w|n dS| dF~/dU_R
     double* blk = nullptr;     // [E][B][B]      P_e, then its LU factors (column-major)
-    int* piv = nullptr;        // [E][B]
+    int* piv = nullptr;        // [E][B] (float32 forms of 2-D levels: GjWork, blocks.cuh)
     // FP32 block path (EMG_PREC_FP32_BLOCKS): float copies of the tables and blocks
     float* vpsi32 = nullptr;
     float* vgw32 = nullptr;
@@ -101,6 +101,8 @@ struct LevelDev {
     float* fjl32 = nullptr;    // [F][QF][25]  face Jacobians for the FP32 blocks
     float* fjr32 = nullptr;    // [F_int][QF][25]
     int gj_variant = 0;        // tuned variant of the FP32 Gauss-Jordan kernel
+    bool gj_split = false;     // 2-D float32 inverses by k_gj_split (blocks that split leave packed)
+    bool asm_plane = false;    // their assembly by k_diag_blocks_pl (the same)
     bool tc_asm = false;       // float32 block assembly on the tensor cores
     bool tc_gj = false;        // float32 block inverse on the tensor cores
 };

@@ -38,7 +38,7 @@ emg_status launch_gj_tc(emg_ctx* c, int B, float* blk, bool* built);
 // differs from the unblocked forms (results agree to float rounding, not bitwise); the
 // variants with different W compute identically.  The inverse is written column-major, as
 // by the other forms.
-// ---- pieces shared by the blocked forms (k_gj_blk, k_gj_la) --------------------------------
+// ---- pieces shared by the blocked forms (k_gj_split, k_gj_blk, k_gj_la) ----------------------
 // Pivot key of row r: the magnitude bits of |a| without their lowest 8 (pivots within 2^-15
 // relative of each other tie), then 255 - r, so that the largest key is a row of (nearly) the
 // largest |a| and, among those, the lowest row; a NaN has magnitude part 0, so any number
@@ -185,33 +185,16 @@ struct GjBlk {
     static constexpr bool VALID = (NB % W == 0) && RS * CS <= 64 && B <= 128;   // piv_pack: rows < 128
 };
 
-template <int B, int W>
-__global__ void __launch_bounds__(32 * W, 16 / W) k_gj_blk(int E, float* __restrict__ blk) {
+// The panels of one block: a[i][j] holds row tx + 32 i, column w + W j, on return the working
+// matrix after all B pivots (row r: row invk[r] of the inverse, column c: its column perm[c]).
+// invk is all -1 on entry.  `beside` runs once in warp 1 while warp 0 factors the first panel.
+template <int B, int W, class Beside>
+__device__ __forceinline__ void gj_blk_panels(float (&a)[GjBlk<B, W>::RS][GjBlk<B, W>::CS], float* Pn, float* Fs,
+                                              float* yw, int* perm, int* invk, int tx, int w, Beside beside) {
     using G = GjBlk<B, W>;
-    constexpr int NB = G::NB, SPW = G::SPW, RS = G::RS, R32 = G::R32, NP = G::NP, CS = G::CS;
-    constexpr int PLD = G::PLD, YL = G::YL, LD = G::LD, T = 32 * W;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    float* tile = reinterpret_cast<float*>(smraw);      // staging (load and store only)
-    float* Pn = tile;                                   // panel columns [R32][PLD]
-    float* Fs = tile + R32 * PLD;                       // factored panel F [R32][PLD]
-    float* Yw = tile + 2 * R32 * PLD;                   // pivot rows, per warp [W][NB][YL]
-    __shared__ int perm[B], invk[R32];
-    const int e = blockIdx.x;
-    const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float* g = blk + (size_t)e * B * B;
-    for (int t = threadIdx.x; t < R32; t += T) invk[t] = -1;
-    for (int t = threadIdx.x; t < B * B; t += T) tile[(t / B) * LD + (t % B)] = g[t];
-    __syncthreads();
-    float a[RS][CS];
-#pragma unroll
-    for (int i = 0; i < RS; ++i)
-#pragma unroll
-        for (int j = 0; j < CS; ++j) {
-            const int r = tx + 32 * i, c = w + W * j;
-            a[i][j] = (r < B && c < B) ? tile[r * LD + c] : 0.0f;
-        }
+    constexpr int NB = G::NB, SPW = G::SPW, RS = G::RS, NP = G::NP, CS = G::CS;
+    constexpr int PLD = G::PLD, YL = G::YL;
     unsigned used = 0u;   // warp 0: bit i set once row tx + 32 i has been a pivot row
-    float* yw = Yw + (size_t)w * NB * YL;
 #pragma unroll 1
     for (int t = 0; t < NP; ++t) {
         const int k0 = t * NB;
@@ -235,6 +218,8 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_gj_blk(int E, float* __restr
             for (int i = 0; i < RS; ++i)
 #pragma unroll
                 for (int c = 0; c < NB; ++c) Fs[(tx + 32 * i) * PLD + c] = x[i][c];
+        } else if (w == 1 && t == 0) {
+            beside();
         }
         __syncthreads();
         // (C) pivot rows of this warp's non-panel columns into the warp's buffer; the pivot
@@ -277,16 +262,144 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_gj_blk(int E, float* __restr
         }
     }
     // NP rotations by SPW = CS slots: every column is back in its own slot
+}
+
+// Every block of the level (list = nullptr, one CTA each), or the blocks that k_gj_split left (list;
+// a few CTAs share them).
+template <int B, int W>
+__global__ void __launch_bounds__(32 * W, 16 / W) k_gj_blk(int E, float* __restrict__ blk, const int* __restrict__ list,
+                                                           int* __restrict__ head) {
+    using G = GjBlk<B, W>;
+    constexpr int RS = G::RS, R32 = G::R32, CS = G::CS, LD = G::LD, T = 32 * W;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float* tile = reinterpret_cast<float*>(smraw);      // staging (load and store only)
+    float* Pn = tile;                                   // panel columns [R32][PLD]
+    float* Fs = tile + R32 * G::PLD;                    // factored panel F [R32][PLD]
+    float* Yw = tile + 2 * R32 * G::PLD;                // pivot rows, per warp [W][NB][YL]
+    __shared__ int perm[B], invk[R32];
+    const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int n = list ? take_list(head) : E;
+#pragma unroll 1
+    for (int it = blockIdx.x; it < n; it += gridDim.x) {
+        float* g = blk + (size_t)(list ? list[it] : it) * B * B;
+        __syncthreads();
+        for (int t = threadIdx.x; t < R32; t += T) invk[t] = -1;
+        for (int t = threadIdx.x; t < B * B; t += T) tile[(t / B) * LD + (t % B)] = g[t];
+        __syncthreads();
+        float a[RS][CS];
+#pragma unroll
+        for (int i = 0; i < RS; ++i)
+#pragma unroll
+            for (int j = 0; j < CS; ++j) {
+                const int r = tx + 32 * i, c = w + W * j;
+                a[i][j] = (r < B && c < B) ? tile[r * LD + c] : 0.0f;
+            }
+        gj_blk_panels<B, W>(a, Pn, Fs, Yw + (size_t)w * G::NB * G::YL, perm, invk, tx, w, []() {});
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < RS; ++i)
+#pragma unroll
+            for (int j = 0; j < CS; ++j) {
+                const int r = tx + 32 * i, c = w + W * j;
+                if (r < B && c < B) tile[perm[c] * LD + invk[r]] = a[i][j];
+            }
+        __syncthreads();
+        for (int t = threadIdx.x; t < B * B; t += T) g[t] = tile[(t / B) * LD + (t % B)];
+    }
+}
+
+// 2-D levels: a block whose spanwise momentum (variable 3) is coupled to no other variable (flow in
+// the plane) splits into systems of 4 N and N unknowns, whose inverses leave packed (blocks.cuh):
+// 0.53 of the multiply-adds and 0.68 of the bytes of the whole block's, and 4 N in place of 5 N
+// pivots in the chain that bounds the kernel (warp 1 inverts the N x N system while warp 0 factors the
+// first panel).  2048 blocks at N = 15: 0.153 ms whole, 0.113 split.  Blocks come packed from the plane assembly (asm_flag) or whole; one that is coupled is
+// left as it is and put on the list for k_gj_blk.
+template <int N, int W>
+struct GjSplit {
+    using G = GjBlk<4 * N, W>;
+    static constexpr int B4 = 4 * N, LD = B4 + 1;
+    static constexpr size_t TILE = (size_t)(B4 * LD + N * N) * sizeof(float);
+    static constexpr size_t WORK = G::WORK + (size_t)N * N * sizeof(float);
+    static constexpr size_t SMEM = ((TILE > WORK ? TILE : WORK) + 15) / 16 * 16;
+    static constexpr bool VALID = G::VALID;
+    static constexpr int MINB = (G::RS * G::CS <= 32 ? 28 : 16) / W;   // 72 or 128 registers a thread
+};
+
+template <int N, int W>
+__global__ void __launch_bounds__(32 * W, GjSplit<N, W>::MINB) k_gj_split(
+    int E, float* __restrict__ blk, const int* __restrict__ asm_flag, int* __restrict__ flag, int* __restrict__ list,
+    int* __restrict__ head) {
+    using S = GjSplit<N, W>;
+    using G = typename S::G;
+    constexpr int B = 5 * N, B4 = 4 * N, LD = S::LD, RS = G::RS, R32 = G::R32, CS = G::CS, T = 32 * W;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float* s3 = reinterpret_cast<float*>(smraw);        // the spanwise block [N][N]
+    float* tile = s3 + N * N;                           // the other variables' (load and store only)
+    float* Yw = reinterpret_cast<float*>(smraw) + (N * N + 3) / 4 * 4;   // pivot rows, per warp [W][NB][YL]
+    float* Pn = Yw + W * G::NB * G::YL;                 // panel columns [R32][PLD]
+    float* Fs = Pn + R32 * G::PLD;                      // factored panel F [R32][PLD]
+    __shared__ int perm[B4], invk[R32], perm3[N], invk3[32];
+    const int tx = threadIdx.x & 31, w = threadIdx.x >> 5, e = blockIdx.x;
+    float* g = blk + (size_t)e * B * B;
+    for (int t = threadIdx.x; t < R32; t += T) invk[t] = -1;
+    if (threadIdx.x < 32) invk3[threadIdx.x] = -1;
+    float* out = blk + gj_packed_at(e, B);
+    bool coupled = false;
+    if (asm_flag && asm_flag[e]) {
+#pragma unroll 8
+        for (int t = threadIdx.x; t < B4 * B4; t += T) tile[t / B4 * LD + t % B4] = out[t];
+        for (int t = threadIdx.x; t < N * N; t += T) s3[t] = out[B4 * B4 + t];
+    } else {
+#pragma unroll 4
+        for (int t = threadIdx.x; t < B * B; t += T) {
+            const int r = t / B, c = t - r * B;
+            const float v = g[t];
+            const int rs = r / N, cs = c / N;
+            if (rs != 3 && cs != 3)
+                tile[(rs == 4 ? r - N : r) * LD + (cs == 4 ? c - N : c)] = v;
+            else if (rs == cs)
+                s3[(r - 3 * N) * N + c - 3 * N] = v;
+            else
+                coupled |= !(v == 0.0f);
+        }
+    }
+    coupled = __syncthreads_or(coupled);
+    if (threadIdx.x == 0) {
+        flag[e] = !coupled;
+        if (coupled) list[atomicAdd(head, 1)] = e;
+    }
+    if (coupled) return;
+    auto spanwise = [&]() {
+        float x[1][N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) x[0][c] = tx < N ? s3[tx * N + c] : 0.0f;
+        unsigned used = 0u;
+        gj_panel_steps<N, 1, N>(x, used, N, 0, tx, perm3, invk3);
+        __syncwarp();
+        if (tx < N)
+#pragma unroll
+            for (int c = 0; c < N; ++c) out[B4 * B4 + perm3[c] * N + invk3[tx]] = x[0][c];
+    };
+    if (W == 1) spanwise();
+    float a[RS][CS];
+#pragma unroll
+    for (int i = 0; i < RS; ++i)
+#pragma unroll
+        for (int j = 0; j < CS; ++j) {
+            const int r = tx + 32 * i, c = w + W * j;
+            a[i][j] = (r < B4 && c < B4) ? tile[r * LD + c] : 0.0f;
+        }
+    gj_blk_panels<B4, W>(a, Pn, Fs, Yw + (size_t)w * G::NB * G::YL, perm, invk, tx, w, spanwise);
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < RS; ++i)
 #pragma unroll
         for (int j = 0; j < CS; ++j) {
             const int r = tx + 32 * i, c = w + W * j;
-            if (r < B && c < B) tile[perm[c] * LD + invk[r]] = a[i][j];
+            if (r < B4 && c < B4) tile[perm[c] * LD + invk[r]] = a[i][j];
         }
     __syncthreads();
-    for (int t = threadIdx.x; t < B * B; t += T) g[t] = tile[(t / B) * LD + (t % B)];
+    for (int t = threadIdx.x; t < B4 * B4; t += T) out[t] = tile[(t / B4) * LD + (t % B4)];
 }
 
 // Look-ahead form of k_gj_blk: warp 0 only factors panels and warps 1..W own the columns
@@ -530,7 +643,7 @@ static cudaError_t gj_blk_go(unsigned E, float* blk, cudaStream_t st) {
         const size_t sm = GjBlk<B, W>::SMEM;
         cudaError_t e = cudaFuncSetAttribute(k_gj_blk<B, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        k_gj_blk<B, W><<<E, 32 * W, sm, st>>>((int)E, blk);
+        k_gj_blk<B, W><<<E, 32 * W, sm, st>>>((int)E, blk, nullptr, nullptr);
         return cudaGetLastError();
     } else {
         return cudaErrorInvalidValue;   // not reached: gj_dispatch checks the variant first
@@ -548,6 +661,52 @@ static cudaError_t gj_la_go(unsigned E, float* blk, cudaStream_t st) {
     } else {
         return cudaErrorInvalidValue;   // not reached: gj_dispatch checks the variant first
     }
+}
+
+// The split form of a 2-D level: kGjBlkWarps[v] warps per element, then the blocks it left (none in
+// plane flow: a few CTAs look at the list's length and end).
+template <int N, int W>
+static cudaError_t gj_split_go(unsigned E, float* blk, const GjWork& k, bool packed, cudaStream_t st) {
+    if constexpr (GjSplit<N, W>::VALID) {
+        const size_t sm = GjSplit<N, W>::SMEM;
+        cudaError_t e = cudaFuncSetAttribute(k_gj_split<N, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        k_gj_split<N, W><<<E, 32 * W, sm, st>>>((int)E, blk, packed ? k.asm_flag : nullptr, k.flag, k.list, k.head);
+        return cudaGetLastError();
+    } else {
+        return cudaErrorInvalidValue;   // not reached: gj_split_valid
+    }
+}
+template <int N>
+static bool gj_split_valid(int v) {
+    return v == 0 ? GjSplit<N, 1>::VALID : v == 1 ? GjSplit<N, 2>::VALID : v == 2 ? GjSplit<N, 4>::VALID : GjSplit<N, 8>::VALID;
+}
+template <int N>
+static cudaError_t gj_split_launch(int v, unsigned E, float* blk, const GjWork& k, bool packed, cudaStream_t st) {
+    cudaError_t e = v == 0   ? gj_split_go<N, 1>(E, blk, k, packed, st)
+                    : v == 1 ? gj_split_go<N, 2>(E, blk, k, packed, st)
+                    : v == 2 ? gj_split_go<N, 4>(E, blk, k, packed, st)
+                             : gj_split_go<N, 8>(E, blk, k, packed, st);
+    if (e != cudaSuccess) return e;
+    using G = GjBlk<5 * N, 4>;
+    static_assert(G::VALID, "the blocked form serves every 2-D block");
+    e = cudaFuncSetAttribute(k_gj_blk<5 * N, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    if (e != cudaSuccess) return e;
+    k_gj_blk<5 * N, 4><<<E < kListBlocks ? E : kListBlocks, 128, G::SMEM, st>>>((int)E, blk, k.list, k.head);
+    return cudaGetLastError();
+}
+// packed: the blocks come from the plane assembly.
+static cudaError_t gj_split_dispatch(int B, int v, unsigned E, float* blk, int* work, bool packed, cudaStream_t st) {
+    const GjWork k = gj_work(work, E);
+    switch (B) {
+        case 15: return gj_split_launch<3>(v, E, blk, k, packed, st);
+        case 30: return gj_split_launch<6>(v, E, blk, k, packed, st);
+        case 50: return gj_split_launch<10>(v, E, blk, k, packed, st);
+        default: return gj_split_launch<15>(v, E, blk, k, packed, st);
+    }
+}
+static bool gj_split_ok(int B, int v) {
+    return B == 15 ? gj_split_valid<3>(v) : B == 30 ? gj_split_valid<6>(v) : B == 50 ? gj_split_valid<10>(v) : gj_split_valid<15>(v);
 }
 
 template <int B>
@@ -605,17 +764,19 @@ static bool gj_valid(int B, int v) {
 }
 
 // Deterministic, diagonally dominant stand-in blocks for timing the variants.
-__global__ void k_fill_tuning_blocks(int64_t n, int B, float* __restrict__ blk) {
+// split: the spanwise momentum's rows and columns coupled to nothing, as in plane flow.
+__global__ void k_fill_tuning_blocks(int64_t n, int B, bool split, float* __restrict__ blk) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n * B * B) return;
     const int c = (int)(t % B), r = (int)((t / B) % B);
     const uint32_t h = (uint32_t)(t * 2654435761ull) ^ (uint32_t)(t >> 13);
-    blk[t] = (r == c ? (float)B : 0.0f) + ((float)(h & 0xffffu) / 65536.0f - 0.5f);
+    const bool zero = split && (r / (B / 5) == 3) != (c / (B / 5) == 3);
+    blk[t] = zero ? 0.0f : (r == c ? (float)B : 0.0f) + ((float)(h & 0xffffu) / 65536.0f - 0.5f);
 }
 
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, bool>, int> g_gj_best;   // (device, B, unblocked asked) -> variant
+std::map<std::tuple<int, int, int>, int> g_gj_best;   // (device, B, family) -> variant
 }  // namespace
 
 // Times every valid variant on min(E, 2048) stand-in blocks per block size of the FP32 levels
@@ -625,17 +786,27 @@ emg_status tune_gj(emg_ctx* c) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     for (int p = 1; p <= c->p_max; ++p) {
         LevelDev& L = c->lv[p];
-        const auto key = std::make_tuple(c->device, L.B, c->prm.block_kernels == 3);
+        // the split form serves 2-D levels unless the tensor-core or unblocked forms are asked for
+        L.gj_split = c->dim == 2 && !L.tc_gj && c->prm.block_kernels != 3;
+        L.asm_plane = L.gj_split && !L.tc_asm && !c->rot;
+        const auto key = std::make_tuple(c->device, L.B, L.gj_split ? 2 : (int)(c->prm.block_kernels == 3));
+        if (L.gj_split)   // the list's length and ticket (piv holds the FP64 form's pivots only)
+            EMG_CUDA_TRY(c, cudaMemsetAsync(L.piv, 0, (size_t)c->E * L.B * sizeof(int), c->stream));
         // the family: blocked where a blocked variant is valid (unless the unblocked forms are
         // asked for), else unblocked
         bool blocked = false;
         if (c->prm.block_kernels != 3)
             for (int v = kGjBlkFirst; v < kGjVariants; ++v) blocked = blocked || gj_valid(L.B, v);
-        const int v_lo = blocked ? kGjBlkFirst : 0, v_hi = blocked ? kGjVariants : kGjBlkFirst;   // 14..21 / 0..13
+        const int v_lo = blocked && !L.gj_split ? kGjBlkFirst : 0;
+        const int v_hi = L.gj_split ? 4 : blocked ? kGjVariants : kGjBlkFirst;   // 0..3 / 14..21 / 0..13
+        auto valid = [&](int v) { return L.gj_split ? gj_split_ok(L.B, v) : gj_valid(L.B, v); };
+        auto name = [&](int v) {
+            return L.gj_split ? "split " + std::to_string(kGjBlkWarps[v]) + " warps" : gj_variant_name(v);
+        };
         if (!c->prm.autotune) {
             L.gj_variant = 0;
             for (int v = v_lo; v < v_hi; ++v)
-                if (gj_valid(L.B, v)) {
+                if (valid(v)) {
                     L.gj_variant = v;
                     break;
                 }
@@ -648,14 +819,15 @@ emg_status tune_gj(emg_ctx* c) {
         auto it = g_gj_best.find(key);
         if (it != g_gj_best.end()) {
             L.gj_variant = it->second;
-            c->tuning += "gj B=" + std::to_string(L.B) + ": " + gj_variant_name(it->second) +
+            c->tuning += "gj B=" + std::to_string(L.B) + ": " + name(it->second) +
                          " (tuned earlier in this process); ";
             continue;
         }
         const int64_t n = std::min<int64_t>(c->E, 2048);
         float* scratch = nullptr;
         EMG_CUDA_TRY(c, cudaMallocAsync((void**)&scratch, (size_t)n * L.B * L.B * sizeof(float), c->stream));
-        k_fill_tuning_blocks<<<(unsigned)((n * L.B * L.B + 255) / 256), 256, 0, c->stream>>>(n, L.B, scratch);
+        const unsigned fill = (unsigned)((n * L.B * L.B + 255) / 256);
+        k_fill_tuning_blocks<<<fill, 256, 0, c->stream>>>(n, L.B, L.gj_split, scratch);
         cudaEvent_t e0, e1;
         EMG_CUDA_TRY(c, cudaEventCreate(&e0));
         EMG_CUDA_TRY(c, cudaEventCreate(&e1));
@@ -663,12 +835,17 @@ emg_status tune_gj(emg_ctx* c) {
         float best_ms = 1e30f;
         std::string note = "gj B=" + std::to_string(L.B) + ":";
         for (int v = v_lo; v < v_hi; ++v) {
-            if (!gj_valid(L.B, v)) continue;
+            if (!valid(v)) continue;
             bool ok = true;
             float ms = 1e30f;
             for (int rep = 0; rep < 3 && ok; ++rep) {
+                if (L.gj_split)   // the inverses left packed are no split blocks
+                    k_fill_tuning_blocks<<<fill, 256, 0, c->stream>>>(n, L.B, true, scratch);
                 EMG_CUDA_TRY(c, cudaEventRecord(e0, c->stream));
-                EMG_CUDA_TRY(c, gj_dispatch(L.B, v, (unsigned)n, scratch, c->stream, &ok));
+                if (L.gj_split)
+                    EMG_CUDA_TRY(c, gj_split_dispatch(L.B, v, (unsigned)n, scratch, L.piv, false, c->stream));
+                else
+                    EMG_CUDA_TRY(c, gj_dispatch(L.B, v, (unsigned)n, scratch, c->stream, &ok));
                 EMG_CUDA_TRY(c, cudaEventRecord(e1, c->stream));
                 EMG_CUDA_TRY(c, cudaEventSynchronize(e1));
                 float t = 0.0f;
@@ -677,7 +854,7 @@ emg_status tune_gj(emg_ctx* c) {
             }
             char buf[64];
             std::snprintf(buf, sizeof(buf), " %.3f ms, ", ms);
-            note += " " + gj_variant_name(v) + buf;
+            note += " " + name(v) + buf;
             if (ms < best_ms) {
                 best_ms = ms;
                 best = v;
@@ -686,9 +863,10 @@ emg_status tune_gj(emg_ctx* c) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         EMG_CUDA_TRY(c, cudaFreeAsync(scratch, c->stream));
+        if (L.gj_split) EMG_CUDA_TRY(c, cudaMemsetAsync(L.piv, 0, (size_t)c->E * L.B * sizeof(int), c->stream));
         g_gj_best[key] = best;
         L.gj_variant = best;
-        c->tuning += note + "-> " + gj_variant_name(best) + "; ";
+        c->tuning += note + "-> " + name(best) + "; ";
     }
     return EMG_OK;
 }
@@ -703,6 +881,12 @@ emg_status launch_lu32(emg_ctx* c, int p) {
     bool ok = true;
     {
         ProfScope _ps(c, PC_LU);
+        if (L.gj_split) {
+            EMG_CUDA_TRY(c, gj_split_dispatch(L.B, L.gj_variant, (unsigned)c->E, L.blk32, L.piv, L.asm_plane, c->stream));
+            ++c->launches;   // two kernels, one counted below
+            EMG_CHECK_LAUNCH(c);
+            return EMG_OK;
+        }
         EMG_CUDA_TRY(c, gj_dispatch(L.B, L.gj_variant, (unsigned)c->E, L.blk32, c->stream, &ok));
     }
     if (!ok) {

@@ -265,8 +265,8 @@ struct DiagRb {
 };
 
 template <int D, int P>
-__global__ void __launch_bounds__(DiagRb<D, P>::THREADS, DiagRb<D, P>::MINB) k_diag_blocks_rb(
-    int E, int nmax, const double* __restrict__ u, const float* __restrict__ vpsi, const float* __restrict__ vgw,
+__device__ __forceinline__ void diag_rb_element(
+    int e, int nmax, const double* __restrict__ u, const float* __restrict__ vpsi, const float* __restrict__ vgw,
     const int* __restrict__ elem_face, const float* __restrict__ fpsiL, const float* __restrict__ fpsiR,
     const float* __restrict__ fjl, const float* __restrict__ fjr, const double* __restrict__ psic,
     const double* __restrict__ hlen, const double* __restrict__ cfl_dev, double g, int shifted,
@@ -286,7 +286,6 @@ __global__ void __launch_bounds__(DiagRb<D, P>::THREADS, DiagRb<D, P>::MINB) k_d
     float(*Us)[5] = reinterpret_cast<float(*)[5]>(smf + R::O_US);
     float(*fjs)[25] = reinterpret_cast<float(*)[25]>(smf + R::O_FJ);
     float* ob = smf;   // over the chunk buffers, once the accumulation is done
-    const int e = blockIdx.x;
     const int tid = threadIdx.x;
     for (int t = tid; t < B; t += blockDim.x) {
         const double v = u[(size_t)e * B + t];
@@ -473,6 +472,23 @@ __global__ void __launch_bounds__(DiagRb<D, P>::THREADS, DiagRb<D, P>::MINB) k_d
     }
 }
 
+// Every element of the level (list = nullptr, one block each), or those that k_diag_blocks_pl left.
+template <int D, int P>
+__global__ void __launch_bounds__(DiagRb<D, P>::THREADS, DiagRb<D, P>::MINB) k_diag_blocks_rb(
+    int E, int nmax, const double* __restrict__ u, const float* __restrict__ vpsi, const float* __restrict__ vgw,
+    const int* __restrict__ elem_face, const float* __restrict__ fpsiL, const float* __restrict__ fpsiR,
+    const float* __restrict__ fjl, const float* __restrict__ fjr, const double* __restrict__ psic,
+    const double* __restrict__ hlen, const double* __restrict__ cfl_dev, double g, int shifted,
+    const double* __restrict__ vvr, float* __restrict__ out, const int* __restrict__ list, int* __restrict__ head) {
+    const int n = list ? take_list(head) : E;
+#pragma unroll 1
+    for (int it = blockIdx.x; it < n; it += gridDim.x) {
+        __syncthreads();
+        diag_rb_element<D, P>(list ? list[it] : it, nmax, u, vpsi, vgw, elem_face, fpsiL, fpsiR, fjl, fjr, psic, hlen,
+                              cfl_dev, g, shifted, vvr, out);
+    }
+}
+
 // Float copies of the level tables used by the FP32 block path.
 __global__ void k_to_float(int64_t n, const double* __restrict__ x, float* __restrict__ y) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -579,6 +595,12 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
     if (!L.tc_asm) {
         // the SIMT (FMA) form of the same contraction
         const int nmax = n_modes(c->dim, c->p_max);
+        const GjWork w = gj_work(L.piv, c->E);
+        if (L.asm_plane) {   // then, below, the elements it left (none in plane flow)
+            st = launch_diag_blocks_plane(c, p, u, cfl_dev, shifted, out);
+            if (st != EMG_OK) return st;
+        }
+        const unsigned grid = L.asm_plane ? (unsigned)std::min<int64_t>(c->E, kListBlocks) : (unsigned)c->E;
 #define EMG_DB32(DD, PP)                                                                                    \
     {                                                                                                       \
         ProfScope _ps(c, PC_DIAG);                                                                          \
@@ -587,9 +609,10 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
                 c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, nullptr, out);                        \
         else                                                                                                \
-            k_diag_blocks_rb<DD, PP><<<(unsigned)c->E, DiagRb<DD, PP>::THREADS, 0, c->stream>>>(            \
+            k_diag_blocks_rb<DD, PP><<<grid, DiagRb<DD, PP>::THREADS, 0, c->stream>>>(                      \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
-                c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, out);                                 \
+                c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, out,                                  \
+                L.asm_plane ? w.asm_list : nullptr, w.asm_head);                                            \
     }
         EMG_DISPATCH_DP(c->dim, p, EMG_DB32)
 #undef EMG_DB32

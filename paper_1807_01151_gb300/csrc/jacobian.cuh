@@ -70,6 +70,9 @@ emg_status launch_face_jacobian32(emg_ctx* c, int p, const double* u);
 emg_status launch_diag_blocks_tc(emg_ctx* c, int p, const double* u, const double* cfl_dev, int shifted,
                                  float* out);
 
+// Float32 assembly of 2-D levels: blocks of plane flow packed, the others on a list (jac_plane.cu).
+emg_status launch_diag_blocks_plane(emg_ctx* c, int p, const double* u, const double* cfl_dev, int shifted, float* out);
+
 // FP64 assembly on the integer pipe (jac_fix.cu): which levels it serves, and its launch (P_e or
 // D_e without the rotating frame's source term).
 bool diag_blocks_fx_serves(int dim, int p);

@@ -358,26 +358,82 @@ __global__ void __launch_bounds__(128) k_stage(int E, const double* __restrict__
 }
 
 // u^(k) = u^n + beta P_e^{-1} r_e with P_e^{-1} column-major: one warp per element, each
-// lane owns rows lane, lane+32, ...; every column is a coalesced read.
-template <int B, class T>
-__global__ void __launch_bounds__(128) k_stage_gemv(int E, const T* __restrict__ inv, const double* __restrict__ r,
-                                                    const double* __restrict__ un, double beta,
-                                                    double* __restrict__ out) {
-    constexpr int RPL = (B + 31) / 32;
-    __shared__ T rs[4][B];
+// lane owns rows lane, lane+32, ...; every column is a coalesced read.  Bound by the bytes of the
+// inverses.  SPLIT (2-D): an element with a packed inverse (blocks.cuh) reads its 16 N^2 floats 16
+// bytes at a time, all loads independent: 32 / N groups of N lanes take the columns in turn, lane q of a
+// group the rows 4 q .. 4 q + 3, and the groups' sums are added at the end; the N x N spanwise part only
+// where r has one.  128 x 64, p = 4: 40 -> 27.5 us a launch (126 MB of inverses).
+template <int B, bool SPLIT>
+__global__ void __launch_bounds__(128) k_stage_gemv(int E, const float* __restrict__ inv, const int* __restrict__ split,
+                                                    const double* __restrict__ r, const double* __restrict__ un,
+                                                    double beta, double* __restrict__ out) {
+    constexpr int RPL = (B + 31) / 32, N = B / 5, B4 = 4 * N;
+    __shared__ __align__(16) float rs[4][(B + 3) / 4 * 4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int e = blockIdx.x * 4 + warp;
     if (e >= E) return;
-    for (int t = lane; t < B; t += 32) rs[warp][t] = (T)r[(size_t)e * B + t];
-    __syncwarp();
-    T acc[RPL];
+    const double* re = r + (size_t)e * B;
+    const double* ue = un + (size_t)e * B;
+    double* oe = out + (size_t)e * B;
+    if (SPLIT && split[e]) {   // uniform over the warp
+        constexpr int G = 32 / (N <= 32 ? N : 32), K = (B4 + G - 1) / G;
+        const float4* M4 = reinterpret_cast<const float4*>(inv + gj_packed_at(e, B));
+        const int q = lane % N, g = lane / N;
+        bool any = false;
+        for (int t = lane; t < B; t += 32) {   // packed order: variables 0, 1, 2, 4, then 3
+            const float v = (float)re[t];
+            any |= t / N == 3 && !(re[t] == 0.0);
+            rs[warp][t < 3 * N ? t : t < B4 ? t + N : t - N] = v;
+        }
+        any = __any_sync(0xffffffffu, any);
+        __syncwarp();
+        float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (g < G) {
+#pragma unroll 10
+            for (int k = 0; k < K; ++k) {
+                const int j = k * G + g;
+                if (B4 % G == 0 || j < B4) {
+                    const float rj = rs[warp][j];
+                    const float4 m = __ldg(M4 + j * N + q);
+                    acc.x = fmaf(m.x, rj, acc.x);
+                    acc.y = fmaf(m.y, rj, acc.y);
+                    acc.z = fmaf(m.z, rj, acc.z);
+                    acc.w = fmaf(m.w, rj, acc.w);
+                }
+            }
+        }
+        float4 sum = acc;
 #pragma unroll
-    for (int t = 0; t < RPL; ++t) acc[t] = (T)0;
-    const T* M = inv + (size_t)e * B * B;
+        for (int h = 1; h < G; ++h) {
+            sum.x += __shfl_sync(0xffffffffu, acc.x, (lane + h * N) & 31);
+            sum.y += __shfl_sync(0xffffffffu, acc.y, (lane + h * N) & 31);
+            sum.z += __shfl_sync(0xffffffffu, acc.z, (lane + h * N) & 31);
+            sum.w += __shfl_sync(0xffffffffu, acc.w, (lane + h * N) & 31);
+        }
+        float s3 = 0.0f;
+        if (any && lane < N) {
+            const float* M3 = reinterpret_cast<const float*>(M4) + B4 * B4;
+#pragma unroll
+            for (int j = 0; j < N; ++j) s3 = fmaf(__ldg(M3 + j * N + lane), rs[warp][B4 + j], s3);
+        }
+        __syncwarp();
+        if (g == 0) *reinterpret_cast<float4*>(&rs[warp][4 * q]) = sum;
+        if (lane < N) rs[warp][B4 + lane] = s3;
+        __syncwarp();
+        for (int t = lane; t < B; t += 32)
+            oe[t] = ue[t] + beta * (double)rs[warp][t < 3 * N ? t : t < B4 ? t + N : t - N];
+        return;
+    }
+    for (int t = lane; t < B; t += 32) rs[warp][t] = (float)re[t];
+    __syncwarp();
+    float acc[RPL];
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) acc[t] = 0.0f;
+    const float* M = inv + (size_t)e * B * B;
 #pragma unroll 4
     for (int j = 0; j < B; ++j) {
-        const T rj = rs[warp][j];
-        const T* col = M + (size_t)j * B;
+        const float rj = rs[warp][j];
+        const float* col = M + (size_t)j * B;
 #pragma unroll
         for (int t = 0; t < RPL; ++t) {
             const int i = lane + 32 * t;
@@ -387,10 +443,9 @@ __global__ void __launch_bounds__(128) k_stage_gemv(int E, const T* __restrict__
 #pragma unroll
     for (int t = 0; t < RPL; ++t) {
         const int i = lane + 32 * t;
-        if (i < B) out[(size_t)e * B + i] = un[(size_t)e * B + i] + beta * (double)acc[t];
+        if (i < B) oe[i] = ue[i] + beta * (double)acc[t];
     }
 }
-
 
 static emg_status lu_dispatch(emg_ctx* c, int B, double* blk, int* piv) {
     const unsigned E = (unsigned)c->E;
@@ -450,7 +505,10 @@ emg_status launch_stage32(emg_ctx* c, int p, const double* r, const double* un, 
 #define EMG_GV_CASE(BB)                                                                                  \
     case BB: {                                                                                           \
         ProfScope _ps(c, PC_STAGE);                                                                      \
-        k_stage_gemv<BB, float><<<(E + 3) / 4, 128, 0, c->stream>>>((int)E, L.blk32, r, un, beta, out);  \
+        if (L.gj_split)                                                                                  \
+            k_stage_gemv<BB, (BB <= 75 && BB != 20)><<<(E + 3) / 4, 128, 0, c->stream>>>((int)E, L.blk32, gj_work(L.piv, E).flag, r, un, beta, out); \
+        else                                                                                             \
+            k_stage_gemv<BB, false><<<(E + 3) / 4, 128, 0, c->stream>>>((int)E, L.blk32, nullptr, r, un, beta, out);                \
     }                                                                                                    \
         EMG_CHECK_LAUNCH(c);                                                                             \
         return EMG_OK;
