@@ -716,23 +716,122 @@ struct Pade13 {
 
 constexpr int PHI_CLUSTER = 8;   // blocks (one per SM) sharing the dense products of k_phi
 
-// C = A B on n x n shared matrices with leading dimension ld, split over the cluster: block
-// r forms a contiguous range of the entries (each entry summed in k order by one thread,
-// as on a single block) and stores it into C of every block of the cluster.  The first
-// barrier keeps the stores from overwriting a C that a slower block still reads.
-__device__ __forceinline__ void smm(const double* A, const double* B, double* C, int n, int ld) {
+// C = A B on n x n shared matrices, split over the cluster: block r forms a contiguous range of the
+// entries (each entry summed in k order by one thread, as on a single block) and stores it into C of
+// every block of the cluster.  No block may still read its C: every product ends with a cluster
+// barrier, so a C that was last read before the previous product's end is free.
+__device__ __forceinline__ void smm(const double* A, const double* B, double* C, int n) {
     cg::cluster_group cl = cg::this_cluster();
     const int nr = (int)cl.num_blocks(), rk = (int)cl.block_rank();
     const int tot = n * n, per = (tot + nr - 1) / nr;
     const int t0 = rk * per, t1 = (t0 + per) < tot ? (t0 + per) : tot;
-    cl.sync();
     for (int t = t0 + (int)threadIdx.x; t < t1; t += (int)blockDim.x) {
-        const int i = t / n, j = t % n;
+        const double *a = A + t / n * n, *b = B + t % n;
         double s = 0.0;
-        for (int k = 0; k < n; ++k) s += A[i * ld + k] * B[k * ld + j];
-        for (int r = 0; r < nr; ++r) cl.map_shared_rank(C, r)[i * ld + j] = s;
+#pragma unroll 8
+        for (int k = 0; k < n; ++k) s = fma(a[k], b[k * n], s);
+        for (int r = 0; r < nr; ++r) cl.map_shared_rank(C, r)[t] = s;
     }
     cl.sync();
+}
+
+// LU factors with partial pivoting of the n x n matrix A in place, by the whole block: multipliers
+// below the diagonal, the reciprocals of U's diagonal in rd, the row order in rid (rid[i]: the row that
+// ended in place i).  Two barriers a column: warp 0 updates the next column and finds its pivot while the
+// other warps update the rest.
+__device__ __forceinline__ void phi_lu(double* A, int n, double* rd, int* rid, int* s_piv) {
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    auto find = [&](int c) {   // the first row of largest |A[r][c]|, r >= c
+        double best = -1.0;
+        int bi = c;
+        for (int r = c + lane; r < n; r += 32) {
+            const double v = fabs(A[r * n + c]);
+            if (v > best) {
+                best = v;
+                bi = r;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ob > best || (ob == best && oi < bi)) {
+                best = ob;
+                bi = oi;
+            }
+        }
+        if (lane == 0) {
+            *s_piv = bi;
+            rd[c] = 1.0 / A[bi * n + c];
+            const int t0 = rid[c];
+            rid[c] = rid[bi];
+            rid[bi] = t0;
+        }
+    };
+    for (int t = tid; t < n; t += nt) rid[t] = t;
+    __syncthreads();
+    if (tid < 32) find(0);
+    __syncthreads();
+    for (int c = 0; c < n; ++c) {
+        const int pr = *s_piv;
+        const double ip = rd[c];
+        // rows c and pr swapped outside column c; column c: the multipliers, row c's entry at pr
+        for (int j = tid; j < n; j += nt) {
+            if (j != c && pr != c) {
+                const double t0 = A[c * n + j];
+                A[c * n + j] = A[pr * n + j];
+                A[pr * n + j] = t0;
+            }
+            if (j > c && j != pr) A[j * n + c] *= ip;
+            if (j == c && pr != c) A[pr * n + c] = A[c * n + c] * ip;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            if (c + 1 < n) {
+                const double u = A[c * n + c + 1];
+                for (int r = c + 1 + lane; r < n; r += 32) A[r * n + c + 1] = fma(-A[r * n + c], u, A[r * n + c + 1]);
+                __syncwarp();
+                find(c + 1);
+            }
+        } else {
+            // 8 x 4 tiles per warp
+            const int w = (tid >> 5) - 1, nw = nt / 32 - 1;
+            for (int r = c + 1 + 8 * w + (lane >> 2); r < n; r += 8 * nw) {
+                const double l = A[r * n + c];
+                for (int j = c + 2 + (lane & 3); j < n; j += 4) A[r * n + j] = fma(-l, A[c * n + j], A[r * n + j]);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Column x of A X = R by one warp with phi_lu's factors, in registers (lane l: rows l + 32 s).
+constexpr int PHI_RS = (MAX_KRYLOV + 2 + 31) / 32;
+__device__ __forceinline__ void phi_solve(const double* A, int n, const double* rd, const int* rid, const double* R,
+                                          int col, double (&y)[PHI_RS]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int s = 0; s < PHI_RS; ++s) y[s] = lane + 32 * s < n ? R[rid[lane + 32 * s] * n + col] : 0.0;
+#pragma unroll
+    for (int sc = 0; sc < PHI_RS; ++sc)
+        for (int c = 32 * sc; c < n && c < 32 * sc + 32; ++c) {
+            const double yc = __shfl_sync(0xffffffffu, y[sc], c & 31);
+#pragma unroll
+            for (int s = sc; s < PHI_RS; ++s) {
+                const int r = lane + 32 * s;
+                if (r > c && r < n) y[s] = fma(-A[r * n + c], yc, y[s]);
+            }
+        }
+#pragma unroll
+    for (int sc = PHI_RS - 1; sc >= 0; --sc)
+        for (int c = (n < 32 * sc + 32 ? n : 32 * sc + 32) - 1; c >= 32 * sc; --c) {
+            const double xc = __shfl_sync(0xffffffffu, y[sc], c & 31) * rd[c];
+#pragma unroll
+            for (int s = 0; s <= sc; ++s) {
+                const int r = lane + 32 * s;
+                if (r < c) y[s] = fma(-A[r * n + c], xc, y[s]);
+                if (r == c) y[s] = xc;
+            }
+        }
 }
 
 // EST = false: y = beta * [exp([[H_k, e1], [0, 0]])]_{0:k, k} with k = sc->m_used (the
@@ -741,10 +840,12 @@ __device__ __forceinline__ void smm(const double* A, const double* B, double* C,
 // process has already ended): X = exp([[H_k, e1, 0], [0, 0, 1], [0, 0, 0]]) holds phi_1(H_k)e1
 // and phi_2(H_k)e1 in its last two columns; when h_{k+1,k} |(phi_2(H_k)e1)_k| <= tol
 // ||phi_1(H_k)e1|| the process ends with k steps (sc->broken = 1).
-// A cluster of PHI_CLUSTER blocks: the dense products (bound by one SM's FP64 rate on a
-// single block) are shared out; the cheap element-wise steps and the small pivoted solve
-// are repeated in every block on its own copies, so every block holds the same matrices
-// and block 0 writes the result.
+// A cluster of PHI_CLUSTER blocks: the dense products (bound by one SM's FP64 rate on a single block)
+// and the solve's columns are shared out; the element-wise steps and the factors of the small matrix are
+// repeated in every block on its own copies.  Block 0 writes the result.
+// Bound by the latency of its chains.  m = 30: 160 -> 70 us with the column norms by a warp, one division
+// a column in place of one a thread, two barriers a column in place of four, the substitutions in
+// registers and one cluster barrier a product in place of two.
 template <bool EST>
 __global__ void __cluster_dims__(PHI_CLUSTER, 1, 1)
     k_phi(int m, int jstep, double tol, const double* __restrict__ H, double* __restrict__ y, Pade13 pc,
@@ -755,8 +856,8 @@ __global__ void __cluster_dims__(PHI_CLUSTER, 1, 1)
     if (k == 0) return;
     // uniform over the cluster: every block reads the same flags written by earlier kernels
     if (EST && (*((volatile int*)&sc->broken) || sc->m_used != k)) return;
-    const int n = EST ? k + 2 : k + 1, ld = n;
-    const int nn = ld * n;
+    const int n = EST ? k + 2 : k + 1;
+    const int nn = n * n;
     double* M = sm;
     double* M2 = M + nn;
     double* M4 = M2 + nn;
@@ -765,25 +866,26 @@ __global__ void __cluster_dims__(PHI_CLUSTER, 1, 1)
     double* T2 = T1 + nn;
     double* U = T2 + nn;
     double* Vv = U + nn;
-    __shared__ double s_norm;
-    __shared__ int s_piv;
+    __shared__ double s_norm, rd[MAX_KRYLOV + 2];
+    __shared__ int s_piv, rid[MAX_KRYLOV + 2];
     for (int t = threadIdx.x; t < nn; t += blockDim.x) {
         const int i = t / n, jj = t % n;
         double v = 0.0;
         if (i < k && jj < k && i <= jj + 1) v = H[(size_t)i * m + jj];   // the Hessenberg band only
         if (i == 0 && jj == k) v = 1.0;
         if (EST && i == k && jj == k + 1) v = 1.0;
-        M[i * ld + jj] = v;
+        M[t] = v;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {   // the largest column sum
         double mx = 0.0;
-        for (int j = 0; j < n; ++j) {
+        for (int j = threadIdx.x; j < n; j += 32) {
             double cs = 0.0;
-            for (int i = 0; i < n; ++i) cs += fabs(M[i * ld + j]);
+            for (int i = 0; i < n; ++i) cs += fabs(M[i * n + j]);
             mx = fmax(mx, cs);
         }
-        s_norm = mx;
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (threadIdx.x == 0) s_norm = mx;
     }
     __syncthreads();
     const double theta13 = 5.371920351148152;
@@ -793,18 +895,19 @@ __global__ void __cluster_dims__(PHI_CLUSTER, 1, 1)
     if (isfinite(s_norm) && s_norm > theta13) s = (int)fmin(ceil(log2(s_norm / theta13)), 1100.0);
     const double sc2 = ldexp(1.0, -s);
     for (int t = threadIdx.x; t < nn; t += blockDim.x) M[t] *= sc2;
-    __syncthreads();
-    smm(M, M, M2, n, ld);
-    smm(M2, M2, M4, n, ld);
-    smm(M4, M2, M6, n, ld);
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();   // every block runs and has its M
+    smm(M, M, M2, n);
+    smm(M2, M2, M4, n);
+    smm(M4, M2, M6, n);
     const double* b = pc.b;
     for (int t = threadIdx.x; t < nn; t += blockDim.x) {
         T1[t] = b[13] * M6[t] + b[11] * M4[t] + b[9] * M2[t];
         T2[t] = b[12] * M6[t] + b[10] * M4[t] + b[8] * M2[t];
     }
     __syncthreads();
-    smm(M6, T1, U, n, ld);   // U = M6 (b13 M6 + b11 M4 + b9 M2)
-    smm(M6, T2, Vv, n, ld);  // V = M6 (b12 M6 + b10 M4 + b8 M2)
+    smm(M6, T1, U, n);   // U = M6 (b13 M6 + b11 M4 + b9 M2)
+    smm(M6, T2, Vv, n);  // V = M6 (b12 M6 + b10 M4 + b8 M2)
     for (int t = threadIdx.x; t < nn; t += blockDim.x) {
         const int i = t / n, j = t % n;
         const double id = (i == j) ? 1.0 : 0.0;
@@ -812,77 +915,30 @@ __global__ void __cluster_dims__(PHI_CLUSTER, 1, 1)
         Vv[t] = Vv[t] + b[6] * M6[t] + b[4] * M4[t] + b[2] * M2[t] + b[0] * id;
     }
     __syncthreads();
-    smm(M, T1, U, n, ld);    // U = M (...)
-    // solve (V - U) X = (V + U); A in T1, RHS/X in T2
+    smm(M, T1, T2, n);   // U = M (...), into T2: a slower block may still read its U
+    // solve (V - U) X = (V + U): A in T1, the right-hand sides in U, X in M2
     for (int t = threadIdx.x; t < nn; t += blockDim.x) {
-        T1[t] = Vv[t] - U[t];
-        T2[t] = Vv[t] + U[t];
+        T1[t] = Vv[t] - T2[t];
+        U[t] = Vv[t] + T2[t];
     }
     __syncthreads();
-    for (int c = 0; c < n; ++c) {
-        if (threadIdx.x < 32) {
-            // pivot: the first row (lowest index) of largest |T1[r][c]|, r >= c, by one warp
-            double best = -1.0;
-            int bi = c;
-            for (int r = c + (int)threadIdx.x; r < n; r += 32) {
-                const double v = fabs(T1[r * ld + c]);
-                if (v > best) {
-                    best = v;
-                    bi = r;
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ob > best || (ob == best && oi < bi)) {
-                    best = ob;
-                    bi = oi;
-                }
-            }
-            if (threadIdx.x == 0) s_piv = bi;
+    phi_lu(T1, n, rd, rid, &s_piv);
+    for (int j = (int)cl.block_rank() + PHI_CLUSTER * ((int)threadIdx.x >> 5); j < n; j += PHI_CLUSTER * ((int)blockDim.x >> 5)) {
+        double x[PHI_RS];
+        phi_solve(T1, n, rd, rid, U, j, x);
+#pragma unroll
+        for (int q = 0; q < PHI_RS; ++q) {
+            const int r = ((int)threadIdx.x & 31) + 32 * q;
+            if (r < n)
+                for (int p = 0; p < PHI_CLUSTER; ++p) cl.map_shared_rank(M2, p)[r * n + j] = x[q];
         }
-        __syncthreads();
-        const int pr = s_piv;
-        if (pr != c)
-            for (int j = threadIdx.x; j < n; j += blockDim.x) {
-                double t0 = T1[c * ld + j];
-                T1[c * ld + j] = T1[pr * ld + j];
-                T1[pr * ld + j] = t0;
-                t0 = T2[c * ld + j];
-                T2[c * ld + j] = T2[pr * ld + j];
-                T2[pr * ld + j] = t0;
-            }
-        __syncthreads();
-        const double ip = 1.0 / T1[c * ld + c];
-        for (int t = threadIdx.x; t < (n - c - 1) * (n + n); t += blockDim.x) {
-            const int r = c + 1 + t / (2 * n);
-            const int j = t % (2 * n);
-            const double l = T1[r * ld + c] * ip;
-            if (j < n) {
-                if (j > c) T1[r * ld + j] -= l * T1[c * ld + j];
-            } else {
-                T2[r * ld + (j - n)] -= l * T2[c * ld + (j - n)];
-            }
-        }
-        __syncthreads();
-        for (int r = c + 1 + threadIdx.x; r < n; r += blockDim.x) T1[r * ld + c] = 0.0;
-        __syncthreads();
     }
-    for (int c = n - 1; c >= 0; --c) {
-        const double ip = 1.0 / T1[c * ld + c];
-        for (int j = threadIdx.x; j < n; j += blockDim.x) T2[c * ld + j] *= ip;
-        __syncthreads();
-        for (int t = threadIdx.x; t < c * n; t += blockDim.x) {
-            const int r = t / n, j = t % n;
-            T2[r * ld + j] -= T1[r * ld + c] * T2[c * ld + j];
-        }
-        __syncthreads();
-    }
-    // squaring: X <- X^2, s times (X in T2)
-    double* X = T2;
-    double* Y = U;
+    cl.sync();
+    // squaring: X <- X^2, s times
+    double* X = M2;
+    double* Y = M4;
     for (int it = 0; it < s; ++it) {
-        smm(X, X, Y, n, ld);
+        smm(X, X, Y, n);
         double* t = X;
         X = Y;
         Y = t;
@@ -891,12 +947,12 @@ __global__ void __cluster_dims__(PHI_CLUSTER, 1, 1)
         if (EST) {
             if (threadIdx.x == 0) {
                 double nrm = 0.0;
-                for (int i = 0; i < k; ++i) nrm += X[i * ld + k] * X[i * ld + k];
-                const double err = H[(size_t)k * m + (k - 1)] * fabs(X[(k - 1) * ld + k + 1]);
+                for (int i = 0; i < k; ++i) nrm += X[i * n + k] * X[i * n + k];
+                const double err = H[(size_t)k * m + (k - 1)] * fabs(X[(k - 1) * n + k + 1]);
                 if (err <= tol * sqrt(nrm)) sc->broken = 1;
             }
         } else {
-            for (int i = threadIdx.x; i < k; i += blockDim.x) y[i] = beta * X[i * ld + k];
+            for (int i = threadIdx.x; i < k; i += blockDim.x) y[i] = beta * X[i * n + k];
         }
     }
 }
