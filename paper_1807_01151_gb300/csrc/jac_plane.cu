@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(160, 4) k_diag_blocks_pl(
             };
             const float2* gq = gs + el * Q * N + i;
             const float4* Aq = A4 + el * (2 * Q + FP) * 4 + a4;
-#pragma unroll 2
+#pragma unroll 1
             for (int q = 0; q < Q; ++q) {
                 const float2 gk = gq[q * N];
                 const float4 A0 = Aq[q * 8], A1 = Aq[q * 8 + 4];
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(160, 4) k_diag_blocks_pl(
                                     fmaf(gk.y, A1.z, gk.x * A0.z), fmaf(gk.y, A1.w, gk.x * A0.w)};
                 add(p + q * NPAD, s);
             }
-#pragma unroll 2
+#pragma unroll 1
             for (int t = 0; t < FP; ++t) {
                 const float pi = p[(Q + t) * NPAD + i];
                 const float4 J = Aq[(2 * Q + t) * 4];
@@ -185,12 +185,12 @@ __global__ void __launch_bounds__(160, 4) k_diag_blocks_pl(
             };
             const float2* gq = gs + el * Q * N + i;
             const float* Aq = A3 + el * (2 * Q + FP);
-#pragma unroll 2
+#pragma unroll 1
             for (int q = 0; q < Q; ++q) {
                 const float2 gk = gq[q * N];
                 add(p + q * NPAD, fmaf(gk.y, Aq[2 * q + 1], gk.x * Aq[2 * q]));
             }
-#pragma unroll 2
+#pragma unroll 1
             for (int t = 0; t < FP; ++t) add(p + (Q + t) * NPAD, p[(Q + t) * NPAD + i] * Aq[2 * Q + t]);
         }
     }

@@ -230,39 +230,58 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
     }
 }
 
-// Register-blocked SIMT form of the float32 assembly (the default float32 form): thread
-// (a, i, jg) accumulates row (a,i) of the block for all five b and the JW columns j of group jg,
-// acc[b][j] += s_b psi_j with s_b = sum_k W d_k psi_i A_k[a][b] formed once per point and
-// reused across the JW columns; every staged basis row is read 16 bytes at a time and
+// Register-blocked SIMT form of the float32 assembly (3-D levels, and the 2-D elements that
+// k_diag_blocks_pl leaves): thread (a, i, jg) accumulates row (a,i) of the block for all five b and the
+// JW columns j of group jg, acc[b][j] += s_b psi_j with s_b = sum_k W d_k psi_i A_k[a][b] formed once
+// per point and reused across the JW columns; every staged basis row is read 16 bytes at a time and
 // broadcast.  Per entry the terms are summed in the order of k_diag_blocks (points in order,
 // then the faces, each product as one FMA), so both forms give bitwise the same blocks.
+//
+// Bound by the issue of the multiply-adds (50 paired ones a point at N = 20) and, with the 100
+// accumulators a thread that make them cheap, by what three blocks an SM can hide: the basis and the flux
+// Jacobians of all points are in shared memory before the sums start, and the weighted gradients and the
+// faces' data come by asynchronous copies one chunk or face ahead, so that the sums never wait for memory
+// (one barrier a chunk in place of four).  A thread's Jacobian entries of a point are four (face: two)
+// 16-byte reads.  13824 hexes, p = 3: 9.3 -> 5.6 ms of assembly per mixed V-cycle.
 template <int D, int P>
 struct DiagRb {
-    static constexpr int N = Lv<D, P>::N;
+    using L = Lv<D, P>;
+    static constexpr int N = L::N, Q = L::Q, QF = L::QF, B = L::B;
     static constexpr int JW = N <= 16 ? ((N + 3) / 4) * 4 : 20;    // columns j per thread
     static constexpr int JG = (N + JW - 1) / JW;                     // column groups
     static constexpr int NPAD = JG * JW;                             // padded basis row
     static constexpr int ROWS = 5 * N;                               // (a, i)
     static constexpr int THREADS = ((ROWS * JG + 31) / 32) * 32;
-    static constexpr int QC = D == 2 ? 36 : 24;                      // volume points per chunk
-    static constexpr int B = Lv<D, P>::B;
-    // the finished block leaves through shared memory: whole when it fits, else one b at a time
-    static constexpr bool WHOLE = (size_t)B * B * sizeof(float) <= 24576;
-    static constexpr int OLD = N + 1;                                // row stride of a b-slab
-    static constexpr int OB = WHOLE ? B * B : ROWS * OLD;
-    // shared memory (floats): the chunk and face buffers, with the output buffer over them
-    static constexpr int Q = Lv<D, P>::Q, QF = Lv<D, P>::QF;
-    static constexpr int O_PS = 0;                                   // [QC][NPAD]
-    static constexpr int O_FPS = O_PS + QC * NPAD;                   // [QF][NPAD]
-    static constexpr int O_GS = O_FPS + QF * NPAD;                   // [QC][D][N]
-    static constexpr int O_AS = O_GS + QC * D * N;                   // [QC][D][25]
-    static constexpr int O_US = O_AS + QC * D * 25;                  // [QC][5]
-    static constexpr int O_FJ = O_US + QC * 5;                       // [QF][25]
-    static constexpr int PHASE = O_FJ + QF * 25;
-    static constexpr int SM = PHASE > OB ? PHASE : OB;
+    static constexpr int QC = 16;                                    // volume points per chunk of gradients
+    static constexpr int AK = D == 2 ? 12 : 16;                      // [k][b] entries of a Jacobian row, padded
+    static constexpr int OLD = B | 1;                                // row stride of the finished block
+    // shared memory (floats); the finished block lies over the tables
+    static constexpr int O_PS = 0;                                   // [Q][NPAD]
+    static constexpr int O_AS = O_PS + Q * NPAD;                     // [Q][5][AK]
+    static constexpr int O_FP = O_AS + Q * 5 * AK;                   // 2 x [QF][NPAD]
+    static constexpr int O_FJ = O_FP + 2 * QF * NPAD;                // 2 x [QF][5][8]
+    static constexpr int O_GS = O_FJ + 2 * QF * 40;                  // 2 x [QC][D][N]
+    static constexpr int O_US = O_GS + 2 * QC * D * N;               // [Q][5]
+    static constexpr int PHASE = O_US + Q * 5;
+    static constexpr int SM = PHASE > B * OLD ? PHASE : B * OLD;
+    static_assert(O_AS % 4 == 0 && O_FP % 4 == 0 && O_FJ % 4 == 0 && O_GS % 4 == 0 && NPAD % 4 == 0, "16-byte reads");
     static constexpr int REGS = 5 * JW > 80 ? 168 : 128;             // register budget per thread
     static constexpr int MINB = (65536 / (THREADS * REGS)) < 1 ? 1 : 65536 / (THREADS * REGS);
+    // bytes per asynchronous copy of a basis row: the rows start on its multiples in every table
+    static constexpr int CP = N % 4 == 0 ? 16 : N % 2 == 0 ? 8 : 4;
 };
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory"); }
 
 template <int D, int P>
 __device__ __forceinline__ void diag_rb_element(
@@ -274,42 +293,96 @@ __device__ __forceinline__ void diag_rb_element(
     using L = Lv<D, P>;
     using R = DiagRb<D, P>;
     constexpr int N = L::N, Q = L::Q, QF = L::QF, B = L::B, NF = L::NF;
-    constexpr int JW = R::JW, JG = R::JG, NPAD = R::NPAD, QC = R::QC;
-    __shared__ double ud[B];
-    __shared__ float us[B];
-    __shared__ __align__(16) float smf[R::SM];
-    __shared__ double s_dtau;
-    float(*ps)[NPAD] = reinterpret_cast<float(*)[NPAD]>(smf + R::O_PS);
-    float(*fps)[NPAD] = reinterpret_cast<float(*)[NPAD]>(smf + R::O_FPS);
-    float(*gs)[D][N] = reinterpret_cast<float(*)[D][N]>(smf + R::O_GS);
-    float(*As)[D][25] = reinterpret_cast<float(*)[D][25]>(smf + R::O_AS);
-    float(*Us)[5] = reinterpret_cast<float(*)[5]>(smf + R::O_US);
-    float(*fjs)[25] = reinterpret_cast<float(*)[25]>(smf + R::O_FJ);
-    float* ob = smf;   // over the chunk buffers, once the accumulation is done
+    constexpr int JW = R::JW, JG = R::JG, NPAD = R::NPAD, QC = R::QC, AK = R::AK, T = R::THREADS;
+    extern __shared__ __align__(16) float smf[];
+    __shared__ double ud[B], Uc[5];
+    __shared__ float us[B], s_idt;
+    float* ps = smf + R::O_PS;
+    float* As = smf + R::O_AS;
+    float* Us = smf + R::O_US;
     const int tid = threadIdx.x;
-    for (int t = tid; t < B; t += blockDim.x) {
+    constexpr int CF = R::CP / 4, NR = N / CF;   // floats per copy, copies per row
+    // gradients of the points of chunk c, into buffer c & 1
+    auto fetch_gradients = [&](int c) {
+        const int q0 = c * QC, nq = Q - q0 < QC ? Q - q0 : QC;
+        float* dst = smf + R::O_GS + (c & 1) * QC * D * N;
+        for (int t = tid; t < D * nq * NR; t += T) {
+            const int row = t / NR, x = t % NR * CF, k = row / nq, q = row % nq;
+            cp_async<R::CP>(dst + (q * D + k) * N + x, vgw + (((size_t)e * D + k) * Q + q0 + q) * N + x);
+        }
+    };
+    // basis traces and face Jacobians of face lf, into buffer lf & 1
+    auto fetch_face = [&](int lf) {
+        const int code = elem_face[(size_t)e * NF + lf];
+        const float* pt = ((code & 1) ? fpsiR : fpsiL) + (size_t)(code >> 1) * QF * N;
+        const float* fj = ((code & 1) ? fjr : fjl) + (size_t)(code >> 1) * QF * 25;
+        float* dp = smf + R::O_FP + (lf & 1) * QF * NPAD;
+        float* dj = smf + R::O_FJ + (lf & 1) * QF * 40;
+        for (int t = tid; t < QF * NR; t += T) cp_async<R::CP>(dp + t / NR * NPAD + t % NR * CF, pt + t * CF);
+        for (int t = tid; t < QF * 25; t += T) cp_async<4>(dj + t / 5 * 8 + t % 5, fj + t);
+    };
+    const float* pg = vpsi + (size_t)e * Q * N;
+    for (int t = tid; t < Q * NR; t += T) cp_async<R::CP>(ps + t / NR * NPAD + t % NR * CF, pg + t * CF);
+    cp_async_commit();
+    fetch_gradients(0);
+    cp_async_commit();
+    // padding of the basis rows (the copies never touch it)
+    if constexpr (NPAD > N) {
+        for (int t = tid; t < Q * (NPAD - N); t += T) ps[t / (NPAD - N) * NPAD + N + t % (NPAD - N)] = 0.0f;
+        for (int t = tid; t < 2 * QF * (NPAD - N); t += T)
+            smf[R::O_FP + t / (NPAD - N) * NPAD + N + t % (NPAD - N)] = 0.0f;
+    }
+    for (int t = tid; t < B; t += T) {
         const double v = u[(size_t)e * B + t];
         ud[t] = v;
         us[t] = (float)v;
     }
+    cp_async_wait<1>();
     __syncthreads();
-    if (tid == 0 && shifted) {
-        double Uc[5];
-        for (int a = 0; a < 5; ++a) {
-            double s = 0.0;
-            for (int i = 0; i < N; ++i) s += ud[a * N + i] * psic[(size_t)e * nmax + i];
-            Uc[a] = s;
+    if (shifted && tid < 5) {   // the state at the cell centre
+        double s = 0.0;
+#pragma unroll 5
+        for (int i = 0; i < N; ++i) s += ud[tid * N + i] * psic[(size_t)e * nmax + i];
+        Uc[tid] = s;
+    }
+    for (int t = T - 1 - tid; t < Q * 5; t += T) {
+        const int q = t / 5, c = t % 5;
+        const float* pq = ps + q * NPAD;
+        float s = 0.0f;
+#pragma unroll 5
+        for (int m = 0; m < N; ++m) s += us[c * N + m] * pq[m];
+        Us[t] = s;
+    }
+    __syncthreads();
+    if (tid == 0) {   // dtau of Eq. x3d
+        float x = 0.0f;
+        if (shifted) {
+            const double ir = 1.0 / Uc[0];
+            const double vx = Uc[1] * ir, vy = Uc[2] * ir, vz = Uc[3] * ir;
+            const double q2 = vx * vx + vy * vy + vz * vz;
+            const double pr = (g - 1.0) * (Uc[4] - 0.5 * Uc[0] * q2);
+            const double cs = sqrt(g * pr * ir);
+            x = (float)(1.0 / (cfl_dev[0] * hlen[e] / ((2 * P + 1) * (sqrt(q2) + cs))));
         }
-        const double ir = 1.0 / Uc[0];
-        const double vx = Uc[1] * ir, vy = Uc[2] * ir, vz = Uc[3] * ir;
-        const double q2 = vx * vx + vy * vy + vz * vz;
-        const double pr = (g - 1.0) * (Uc[4] - 0.5 * Uc[0] * q2);
-        const double cs = sqrt(g * pr * ir);
-        s_dtau = cfl_dev[0] * hlen[e] / ((2 * P + 1) * (sqrt(q2) + cs));
+        s_idt = x;
+    }
+    for (int t = T - 1 - tid; t < Q * D; t += T) {
+        const int q = t / D, k = t % D;
+        float A[25];
+        flux_jac_k(Us + q * 5, (float)g, k, A);
+        if (vvr) {   // rotating frame: A_k - (v_r)_k I
+            const float vr = (float)vvr[((size_t)e * Q + q) * 3 + k];
+#pragma unroll
+            for (int a = 0; a < 5; ++a) A[a * 6] -= vr;
+        }
+#pragma unroll
+        for (int a = 0; a < 5; ++a)
+#pragma unroll
+            for (int b = 0; b < 5; ++b) As[(q * 5 + a) * AK + k * 5 + b] = A[a * 5 + b];
     }
     // thread (a, i, jg): consecutive threads take consecutive i, so a warp shares a and jg
     const bool active = tid < R::ROWS * JG;
-    const int a = tid / (N * JG), rem = tid % (N * JG);
+    const int a = active ? tid / (N * JG) : 0, rem = tid % (N * JG);
     const int jg = rem / N, i = rem % N;
     const int j0 = jg * JW;
     float acc[5][JW];
@@ -317,159 +390,89 @@ __device__ __forceinline__ void diag_rb_element(
     for (int b = 0; b < 5; ++b)
 #pragma unroll
         for (int j = 0; j < JW; ++j) acc[b][j] = 0.0f;
-    // face data (basis traces and the signed face Jacobians) of the next face, loaded into
-    // registers one face ahead so that the loads overlap the previous face's (or, for the
-    // first face, the volume's) accumulation; stored to shared memory between two barriers
-    constexpr int T = R::THREADS;
-    constexpr int NPF = (QF * NPAD + T - 1) / T, NJF = (QF * 25 + T - 1) / T;
-    float pf[NPF], pj[NJF];
-    auto fetch_face = [&](int lf) {
-        const int code = elem_face[(size_t)e * NF + lf];
-        const float* pt = ((code & 1) ? fpsiR : fpsiL) + ((size_t)(code >> 1) * QF) * N;
-        const float* fj = ((code & 1) ? fjr : fjl) + ((size_t)(code >> 1) * QF) * 25;
+    auto add = [&](const float* prow, const float (&s)[5]) {
 #pragma unroll
-        for (int k = 0; k < NPF; ++k) {
-            const int t = tid + k * T, q = t / NPAD, j = t % NPAD;
-            pf[k] = (t < QF * NPAD && j < N) ? pt[q * N + j] : 0.0f;
-        }
+        for (int jj = 0; jj < JW; jj += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(prow + j0 + jj);
 #pragma unroll
-        for (int k = 0; k < NJF; ++k) {
-            const int t = tid + k * T;
-            pj[k] = t < QF * 25 ? ((code & 1) ? fj[t] : -fj[t]) : 0.0f;
+            for (int b = 0; b < 5; ++b) {
+                fma2f(s[b], v.x, v.y, acc[b][jj], acc[b][jj + 1]);
+                fma2f(s[b], v.z, v.w, acc[b][jj + 2], acc[b][jj + 3]);
+            }
         }
     };
-    fetch_face(0);
-    if (P > 0) {
-        for (int q0 = 0; q0 < Q; q0 += QC) {
-            const int nq = (Q - q0) < QC ? (Q - q0) : QC;
-            __syncthreads();
-            const float* pg = vpsi + ((size_t)e * Q + q0) * N;
-            for (int t = tid; t < nq * NPAD; t += blockDim.x) {
-                const int q = t / NPAD, j = t % NPAD;
-                ps[q][j] = j < N ? pg[q * N + j] : 0.0f;
-            }
-            for (int t = tid; t < D * nq * N; t += blockDim.x) {
-                const int k = t / (nq * N), r = t % (nq * N);
-                gs[r / N][k][r % N] = vgw[(((size_t)e * D + k) * Q + q0) * N + r];
-            }
-            for (int t = tid; t < nq * 5; t += blockDim.x) {
-                const int q = t / 5, c = t % 5;
-                const float* pq = pg + (size_t)q * N;
-                float s = 0.0f;
-                for (int m = 0; m < N; ++m) s += us[c * N + m] * pq[m];
-                Us[q][c] = s;
-            }
-            __syncthreads();
-            for (int t = tid; t < nq * D; t += blockDim.x) {
-                flux_jac_k(Us[t / D], (float)g, t % D, As[t / D][t % D]);
-                if (vvr) {   // rotating frame: A_k - (v_r)_k I
-                    const float vr = (float)vvr[((size_t)e * Q + q0 + t / D) * 3 + t % D];
-#pragma unroll
-                    for (int a = 0; a < 5; ++a) As[t / D][t % D][a * 6] -= vr;
-                }
-            }
-            __syncthreads();
-            if (active) {
+    constexpr int NCH = (Q + QC - 1) / QC;
 #pragma unroll 1
-                for (int t = 0; t < nq; ++t) {
-                    float gk[D];
+    for (int c = 0; c < NCH; ++c) {
+        cp_async_wait<0>();
+        __syncthreads();   // chunk c is in; every thread has finished chunk c - 1, whose buffer is free
+        if (c + 1 < NCH)
+            fetch_gradients(c + 1);
+        else
+            fetch_face(0);
+        cp_async_commit();
+        if (active) {
+            const int q0 = c * QC, nq = Q - q0 < QC ? Q - q0 : QC;
+            const float* gq = smf + R::O_GS + (c & 1) * QC * D * N + i;
+#pragma unroll 1
+            for (int t = 0; t < nq; ++t) {
+                const float4* Aq = reinterpret_cast<const float4*>(As + ((q0 + t) * 5 + a) * AK);
+                float A[AK];
 #pragma unroll
-                    for (int k = 0; k < D; ++k) gk[k] = gs[t][k][i];
-                    float s[5];
-#pragma unroll
-                    for (int b = 0; b < 5; ++b) {
-                        float x = 0.0f;
-#pragma unroll
-                        for (int k = 0; k < D; ++k) x += gk[k] * As[t][k][a * 5 + b];
-                        s[b] = x;
-                    }
-#pragma unroll
-                    for (int jj = 0; jj < JW; jj += 4) {
-                        const float4 v = *reinterpret_cast<const float4*>(&ps[t][j0 + jj]);
-                        const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                        for (int c = 0; c < 4; c += 2)
-#pragma unroll
-                            for (int b = 0; b < 5; ++b) fma2f(s[b], vv[c], vv[c + 1], acc[b][jj + c], acc[b][jj + c + 1]);
-                    }
+                for (int x = 0; x < AK; x += 4) {
+                    const float4 v = Aq[x / 4];
+                    A[x] = v.x, A[x + 1] = v.y, A[x + 2] = v.z, A[x + 3] = v.w;
                 }
+                float s[5];
+#pragma unroll
+                for (int b = 0; b < 5; ++b) s[b] = 0.0f;
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    const float gk = gq[(t * D + k) * N];
+#pragma unroll
+                    for (int b = 0; b < 5; ++b) s[b] += gk * A[k * 5 + b];
+                }
+                add(ps + (q0 + t) * NPAD, s);
             }
         }
     }
 #pragma unroll 1
     for (int lf = 0; lf < NF; ++lf) {
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < NPF; ++k) {
-            const int t = tid + k * T;
-            if (t < QF * NPAD) fps[t / NPAD][t % NPAD] = pf[k];
-        }
-#pragma unroll
-        for (int k = 0; k < NJF; ++k) {
-            const int t = tid + k * T;
-            if (t < QF * 25) fjs[t / 25][t % 25] = pj[k];
-        }
+        cp_async_wait<0>();
         __syncthreads();
         if (lf + 1 < NF) fetch_face(lf + 1);
+        cp_async_commit();
         if (active) {
+            // the R side enters with the sign +, the L side with -
+            const float sg = (elem_face[(size_t)e * NF + lf] & 1) ? 1.0f : -1.0f;
+            const float* fp = smf + R::O_FP + (lf & 1) * QF * NPAD;
+            const float* fj = smf + R::O_FJ + (lf & 1) * QF * 40 + a * 8;
 #pragma unroll 1
             for (int t = 0; t < QF; ++t) {
-                const float pi = fps[t][i];
-                float s[5];
-#pragma unroll
-                for (int b = 0; b < 5; ++b) s[b] = pi * fjs[t][a * 5 + b];
-#pragma unroll
-                for (int jj = 0; jj < JW; jj += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(&fps[t][j0 + jj]);
-                    const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                    for (int c = 0; c < 4; c += 2)
-#pragma unroll
-                        for (int b = 0; b < 5; ++b) fma2f(s[b], vv[c], vv[c + 1], acc[b][jj + c], acc[b][jj + c + 1]);
-                }
+                const float pi = sg * fp[t * NPAD + i];
+                const float4 J = *reinterpret_cast<const float4*>(fj + t * 40);
+                const float s[5] = {pi * J.x, pi * J.y, pi * J.z, pi * J.w, pi * fj[t * 40 + 4]};
+                add(fp + t * NPAD, s);
             }
         }
     }
-    const float idt = shifted ? (float)(1.0 / s_dtau) : 0.0f;
+    __syncthreads();
+    if (active) {
+        const float idt = s_idt;
+        float* o = smf + (a * N + i) * R::OLD + j0;
+#pragma unroll
+        for (int b = 0; b < 5; ++b)
+#pragma unroll
+            for (int j = 0; j < JW; ++j)
+                if (j0 + j < N) {
+                    const float v = acc[b][j];
+                    o[b * N + j] = shifted ? ((a == b && i == j0 + j) ? idt : 0.0f) - v : v;
+                }
+    }
+    __syncthreads();
     float* g_out = out + (size_t)e * B * B;
-    if (R::WHOLE) {
-        __syncthreads();
-        if (active) {
-#pragma unroll
-            for (int b = 0; b < 5; ++b)
-#pragma unroll
-                for (int j = 0; j < JW; ++j) {
-                    const int jj = j0 + j;
-                    if (jj < N) {
-                        const float v = acc[b][j];
-                        ob[(a * N + i) * B + b * N + jj] = shifted ? ((a == b && i == jj) ? idt : 0.0f) - v : v;
-                    }
-                }
-        }
-        __syncthreads();
-        for (int t = tid; t < B * B; t += blockDim.x) g_out[t] = ob[t];
-    } else {
-        constexpr int OLD = R::OLD;
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {   // unrolled: acc[b] stays in registers
-            __syncthreads();
-            if (active) {
-#pragma unroll
-                for (int j = 0; j < JW; ++j) {
-                    const int jj = j0 + j;
-                    if (jj < N) {
-                        const float v = acc[b][j];
-                        ob[(a * N + i) * OLD + jj] = shifted ? ((a == b && i == jj) ? idt : 0.0f) - v : v;
-                    }
-                }
-            }
-            __syncthreads();
-            for (int t = tid; t < R::ROWS * N; t += blockDim.x) {
-                const int r = t / N, j = t % N;
-                g_out[(size_t)r * B + b * N + j] = ob[r * OLD + j];
-            }
-        }
-    }
+#pragma unroll 4
+    for (int t = tid; t < B * B; t += T) g_out[t] = smf[t / B * R::OLD + t % B];
 }
 
 // Every element of the level (list = nullptr, one block each), or those that k_diag_blocks_pl left.
@@ -602,14 +605,16 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
         }
         const unsigned grid = L.asm_plane ? (unsigned)std::min<int64_t>(c->E, kListBlocks) : (unsigned)c->E;
 #define EMG_DB32(DD, PP)                                                                                    \
-    {                                                                                                       \
+    if constexpr (PP > 0) {                                                                                 \
+        EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_diag_blocks_rb<DD, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                             DiagRb<DD, PP>::SM * 4));                                      \
         ProfScope _ps(c, PC_DIAG);                                                                          \
         if (c->prm.block_kernels == 3)                                                                      \
             k_diag_blocks<DD, PP, float><<<(unsigned)c->E, DiagCfg<DD, PP>::THREADS, 0, c->stream>>>(       \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
                 c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, nullptr, out);                        \
         else                                                                                                \
-            k_diag_blocks_rb<DD, PP><<<grid, DiagRb<DD, PP>::THREADS, 0, c->stream>>>(                      \
+            k_diag_blocks_rb<DD, PP><<<grid, DiagRb<DD, PP>::THREADS, DiagRb<DD, PP>::SM * 4, c->stream>>>( \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
                 c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, out,                                  \
                 L.asm_plane ? w.asm_list : nullptr, w.asm_head);                                            \

@@ -43,10 +43,9 @@ __device__ __forceinline__ void flux_jac_k(const float U[5], float g, int k, flo
     const float a0 = 0.5f * (g - 1.0f) * q2;
     const float p = (g - 1.0f) * (U[4] - 0.5f * U[0] * q2);
     const float H = (U[4] + p) * ir;
-    const float vk = v[k];
+    const float vk = k == 0 ? v[0] : k == 1 ? v[1] : v[2];   // no index that is not known when compiling: A stays in registers
 #pragma unroll
-    for (int t = 0; t < 25; ++t) A[t] = 0.0f;
-    A[1 + k] = 1.0f;
+    for (int t = 0; t < 25; ++t) A[t] = t == 1 + k ? 1.0f : 0.0f;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
         float* row = A + 5 * (1 + m);
