@@ -38,42 +38,44 @@ emg_status launch_gj_tc(emg_ctx* c, int B, float* blk, bool* built);
 // differs from the unblocked forms (results agree to float rounding, not bitwise); the
 // variants with different W compute identically.  The inverse is written column-major, as
 // by the other forms.
-// ---- pieces shared by the blocked forms (k_gj_split, k_gj_blk, k_gj_la) ----------------------
+// ---- pieces shared by the blocked forms (k_gj_split, k_gj_blk) ----------------------
 // Pivot key of row r: the magnitude bits of |a| without their lowest 8 (pivots within 2^-15
 // relative of each other tie), then 255 - r, so that the largest key is a row of (nearly) the
-// largest |a| and, among those, the lowest row; a NaN has magnitude part 0, so any number
-// beats it and a column without a number yields its lowest unused row.  Rows r < 128.
-__device__ __forceinline__ unsigned piv_pack(float x, int r) {
-    const unsigned k = (unsigned)(piv_key(x) + 1);   // 0 for NaN
-    return ((k >> 8) << 8) | (unsigned)(255 - r);
-}
+// largest |a| and, among those, the lowest row; a NaN wins (the inverse of such a block is NaN).  One
+// logic operation with the row's mask: 0 for a row that has been taken (or is none), so the key of every
+// row left is larger.  Rows r < 128.
+__device__ __forceinline__ unsigned piv_mask(int r, int B) { return r < B ? 0x7fffff00u | (unsigned)(255 - r) : 0u; }
+__device__ __forceinline__ unsigned piv_pack(float x, unsigned mask) { return (__float_as_uint(x) | 0x800000ffu) & mask; }
 
 // The in-place Gauss-Jordan steps of a panel of NB columns held by one warp (lane tx: rows
 // tx + 32 i, x[i][c] for panel column c), one warp reduction per pivot: pivot rows are
-// recorded in perm[k0 + s] and their steps in invk[p] = k0 + s; `used` marks this lane's rows
-// already taken.
+// recorded in perm[k0 + s] and their steps in invk[p] = k0 + s; mask: the rows' key masks.  Bound by
+// the latency of the chain pivot search, broadcast, reciprocal, update: the next column is updated and
+// its pivot searched before the other columns' updates are issued, and a key is one operation.  2048
+// blocks: B = 100 0.392 -> 0.354 ms, B = 75 split 0.132 -> 0.107 ms, B = 50 0.061 -> 0.053 ms.
 template <int B, int RS, int NB>
-__device__ __forceinline__ void gj_panel_steps(float (&x)[RS][NB], unsigned& used, int nb, int k0, int tx, int* perm,
+__device__ __forceinline__ void gj_panel_steps(float (&x)[RS][NB], unsigned (&mask)[RS], int nb, int k0, int tx, int* perm,
                                                int* invk) {
+    auto search = [&](int s) {
+        unsigned km = piv_pack(x[0][s], mask[0]);
+#pragma unroll
+        for (int i = 1; i < RS; ++i) km = max(km, piv_pack(x[i][s], mask[i]));
+        return __reduce_max_sync(0xffffffffu, km);
+    };
+    unsigned km = search(0);
 #pragma unroll
     for (int s = 0; s < NB; ++s) {
         if (s >= nb) break;   // uniform
-        unsigned km = 0u;
-#pragma unroll
-        for (int i = 0; i < RS; ++i) {
-            const int r = tx + 32 * i;
-            const unsigned kk = (r < B && !((used >> i) & 1u)) ? piv_pack(x[i][s], r) : 0u;
-            km = kk > km ? kk : km;
-        }
-        km = __reduce_max_sync(0xffffffffu, km);
         const int p = 255 - (int)(km & 255u);
         const int pl = p & 31, pi = p >> 5;
         float rk[NB];
 #pragma unroll
         for (int ii = 0; ii < RS; ++ii)
             if (pi == ii) {   // warp-uniform branch
+                rk[s] = __shfl_sync(0xffffffffu, x[ii][s], pl);
 #pragma unroll
-                for (int c = 0; c < NB; ++c) rk[c] = __shfl_sync(0xffffffffu, x[ii][c], pl);
+                for (int c = 0; c < NB; ++c)
+                    if (c != s) rk[c] = __shfl_sync(0xffffffffu, x[ii][c], pl);
             }
         const float inv = __frcp_rn(rk[s]);   // correctly rounded, as 1.0f / rk[s]
 #pragma unroll
@@ -81,24 +83,30 @@ __device__ __forceinline__ void gj_panel_steps(float (&x)[RS][NB], unsigned& use
         float f[RS];
 #pragma unroll
         for (int i = 0; i < RS; ++i) {
-            f[i] = (tx + 32 * i == p) ? 0.0f : x[i][s];
+            f[i] = -x[i][s];
             x[i][s] = 0.0f;
+            if (tx + 32 * i == p) mask[i] = 0u;
         }
+        // columns c0, c0 + 1 (or the odd last one) of every row; the pivot row is scaled instead
+        auto update = [&](int c0) {
 #pragma unroll
-        for (int i = 0; i < RS; ++i) {
-#pragma unroll
-            for (int c = 0; c + 1 < NB; c += 2) fma2f(-f[i], rk[c], rk[c + 1], x[i][c], x[i][c + 1]);
-            if (NB % 2) x[i][NB - 1] = fmaf(-f[i], rk[NB - 1], x[i][NB - 1]);
-        }
-        if (tx == pl) {
-            used |= 1u << pi;
-#pragma unroll
-            for (int ii = 0; ii < RS; ++ii)
-                if (pi == ii) {
-#pragma unroll
-                    for (int c = 0; c < NB; ++c) x[ii][c] = rk[c];
+            for (int i = 0; i < RS; ++i) {
+                if (c0 + 1 < NB)
+                    fma2f(f[i], rk[c0], rk[c0 + 1], x[i][c0], x[i][c0 + 1]);
+                else
+                    x[i][c0] = fmaf(f[i], rk[c0], x[i][c0]);
+                if (tx + 32 * i == p) {
+                    x[i][c0] = rk[c0];
+                    if (c0 + 1 < NB) x[i][c0 + 1] = rk[c0 + 1];
                 }
-        }
+            }
+        };
+        const int first = s + 1 < NB ? (s + 1) / 2 * 2 : 0;
+        update(first);
+        if (s + 1 < NB) km = search(s + 1);
+#pragma unroll
+        for (int c = 0; c < NB; c += 2)
+            if (c != first) update(c);
         if (tx == 0) {
             perm[k0 + s] = p;
             invk[p] = k0 + s;
@@ -182,7 +190,9 @@ struct GjBlk {
     static constexpr size_t TILE = (size_t)B * LD * sizeof(float);
     static constexpr size_t WORK = (size_t)(2 * R32 * PLD + W * NB * YL) * sizeof(float);
     static constexpr size_t SMEM = ((TILE > WORK ? TILE : WORK) + 15) / 16 * 16;
-    static constexpr bool VALID = (NB % W == 0) && RS * CS <= 64 && B <= 128;   // piv_pack: rows < 128
+    static constexpr int MAXV = W == 1 ? 128 : 64;      // values a thread holds
+    static constexpr bool VALID = (NB % W == 0) && RS * CS <= MAXV && B <= 128;   // piv_pack: rows < 128
+    static constexpr int MINB = RS * CS > 96 ? 10 : RS * CS > 64 ? 12 : 16 / W;
 };
 
 // The panels of one block: a[i][j] holds row tx + 32 i, column w + W j, on return the working
@@ -194,7 +204,9 @@ __device__ __forceinline__ void gj_blk_panels(float (&a)[GjBlk<B, W>::RS][GjBlk<
     using G = GjBlk<B, W>;
     constexpr int NB = G::NB, SPW = G::SPW, RS = G::RS, NP = G::NP, CS = G::CS;
     constexpr int PLD = G::PLD, YL = G::YL;
-    unsigned used = 0u;   // warp 0: bit i set once row tx + 32 i has been a pivot row
+    unsigned used[RS];   // warp 0: key masks of its rows
+#pragma unroll
+    for (int i = 0; i < RS; ++i) used[i] = piv_mask(tx + 32 * i, B);
 #pragma unroll 1
     for (int t = 0; t < NP; ++t) {
         const int k0 = t * NB;
@@ -267,7 +279,7 @@ __device__ __forceinline__ void gj_blk_panels(float (&a)[GjBlk<B, W>::RS][GjBlk<
 // Every block of the level (list = nullptr, one CTA each), or the blocks that k_gj_split left (list;
 // a few CTAs share them).
 template <int B, int W>
-__global__ void __launch_bounds__(32 * W, 16 / W) k_gj_blk(int E, float* __restrict__ blk, const int* __restrict__ list,
+__global__ void __launch_bounds__(32 * W, GjBlk<B, W>::MINB) k_gj_blk(int E, float* __restrict__ blk, const int* __restrict__ list,
                                                            int* __restrict__ head) {
     using G = GjBlk<B, W>;
     constexpr int RS = G::RS, R32 = G::R32, CS = G::CS, LD = G::LD, T = 32 * W;
@@ -312,7 +324,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_gj_blk(int E, float* __restr
 // the plane) splits into systems of 4 N and N unknowns, whose inverses leave packed (blocks.cuh):
 // 0.53 of the multiply-adds and 0.68 of the bytes of the whole block's, and 4 N in place of 5 N
 // pivots in the chain that bounds the kernel (warp 1 inverts the N x N system while warp 0 factors the
-// first panel).  2048 blocks at N = 15: 0.153 ms whole, 0.113 split.  Blocks come packed from the plane assembly (asm_flag) or whole; one that is coupled is
+// first panel).  2048 blocks at N = 15: 0.153 ms whole, 0.107 split.  Blocks come packed from the plane assembly (asm_flag) or whole; one that is coupled is
 // left as it is and put on the list for k_gj_blk.
 template <int N, int W>
 struct GjSplit {
@@ -322,7 +334,7 @@ struct GjSplit {
     static constexpr size_t WORK = G::WORK + (size_t)N * N * sizeof(float);
     static constexpr size_t SMEM = ((TILE > WORK ? TILE : WORK) + 15) / 16 * 16;
     static constexpr bool VALID = G::VALID;
-    static constexpr int MINB = (G::RS * G::CS <= 32 ? 28 : 16) / W;   // 72 or 128 registers a thread
+    static constexpr int MINB = W > 1 && G::RS * G::CS <= 32 ? 28 / W : G::MINB;
 };
 
 template <int N, int W>
@@ -373,7 +385,7 @@ __global__ void __launch_bounds__(32 * W, GjSplit<N, W>::MINB) k_gj_split(
         float x[1][N];
 #pragma unroll
         for (int c = 0; c < N; ++c) x[0][c] = tx < N ? s3[tx * N + c] : 0.0f;
-        unsigned used = 0u;
+        unsigned used[1] = {piv_mask(tx, N)};
         gj_panel_steps<N, 1, N>(x, used, N, 0, tx, perm3, invk3);
         __syncwarp();
         if (tx < N)
@@ -402,195 +414,13 @@ __global__ void __launch_bounds__(32 * W, GjSplit<N, W>::MINB) k_gj_split(
     for (int t = threadIdx.x; t < B4 * B4; t += T) out[t] = tile[(t / B4) * LD + (t % B4)];
 }
 
-// Look-ahead form of k_gj_blk: warp 0 only factors panels and warps 1..W own the columns
-// (column c: warp 1 + c mod W, slot c / W).  At panel t the update warps first bring panel
-// t+1's columns up to date and hand them to warp 0, then update the remaining columns, so the
-// factorisation of panel t+1 runs while the trailing update of panel t is still going on.
-// Two named barriers carry the hand-offs (panel ready: the update warps arrive, warp 0 waits;
-// factor ready: warp 0 arrives, the update warps wait); panel and factor buffers are double
-// buffered.  Every entry receives the multiply-adds of k_gj_blk in the same order, and the
-// panel steps are those of k_gj_blk: bitwise the same inverse.
-template <int B, int W>
-struct GjLa {
-    static constexpr int NB = 8;
-    static constexpr int SPW = NB / W;
-    static constexpr int RS = (B + 31) / 32;
-    static constexpr int R32 = 32 * RS;
-    static constexpr int NP = (B + NB - 1) / NB;
-    static constexpr int CS = NP * SPW;
-    static constexpr int PLD = NB + 1;
-    static constexpr int YN = CS - SPW;
-    static constexpr int YL = YN > 0 ? ((YN + 3) / 4) * 4 : 4;
-    static constexpr int LD = (B % 2) ? B + 2 : B + 1;
-    static constexpr int THREADS = 32 * (W + 1);
-    static constexpr size_t TILE = (size_t)B * LD * sizeof(float);
-    static constexpr size_t WORK = (size_t)(4 * R32 * PLD + W * NB * YL) * sizeof(float);
-    static constexpr size_t SMEM = ((TILE > WORK ? TILE : WORK) + 15) / 16 * 16;
-    static constexpr bool VALID = (NB % W == 0) && RS * CS <= 64 && NP >= 2 && B <= 128;
-};
-
-__device__ __forceinline__ void named_sync(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-__device__ __forceinline__ void named_arrive(int id, int count) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
-template <int B, int W>
-__global__ void __launch_bounds__(32 * (W + 1)) k_gj_la(int E, float* __restrict__ blk) {
-    using G = GjLa<B, W>;
-    constexpr int NB = G::NB, SPW = G::SPW, RS = G::RS, R32 = G::R32, NP = G::NP, CS = G::CS;
-    constexpr int PLD = G::PLD, YL = G::YL, LD = G::LD, T = G::THREADS;
-    constexpr int BAR_PANEL = 1, BAR_F = 2;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    float* tile = reinterpret_cast<float*>(smraw);      // staging (load and store only)
-    float* Pn = tile;                                   // 2 x [R32][PLD] panel columns
-    float* Fs = tile + 2 * R32 * PLD;                   // 2 x [R32][PLD] factored panels
-    float* Yw = tile + 4 * R32 * PLD;                   // [W][NB][YL] pivot rows per update warp
-    __shared__ int perm[B], invk[R32];
-    const int e = blockIdx.x;
-    const int tx = threadIdx.x & 31, wq = threadIdx.x >> 5, w = wq - 1;
-    float* g = blk + (size_t)e * B * B;
-    for (int t = threadIdx.x; t < R32; t += T) invk[t] = -1;
-    for (int t = threadIdx.x; t < B * B; t += T) tile[(t / B) * LD + (t % B)] = g[t];
-    __syncthreads();
-    float a[RS][CS];
-    if (wq > 0) {
-#pragma unroll
-        for (int i = 0; i < RS; ++i)
-#pragma unroll
-            for (int j = 0; j < CS; ++j) {
-                const int r = tx + 32 * i, c = w + W * j;
-                a[i][j] = (r < B && c < B) ? tile[r * LD + c] : 0.0f;
-            }
-    }
-    __syncthreads();   // the staging tile becomes the work buffers
-    if (wq == 0) {
-        // ---- factor warp -----------------------------------------------------------------
-        unsigned used = 0u;
-#pragma unroll 1
-        for (int t = 0; t < NP; ++t) {
-            const int k0 = t * NB;
-            const int nb = (B - k0) < NB ? (B - k0) : NB;
-            const float* pn = Pn + (t & 1) * R32 * PLD;
-            float* fs = Fs + (t & 1) * R32 * PLD;
-            named_sync(BAR_PANEL, T);
-            float x[RS][NB];
-#pragma unroll
-            for (int i = 0; i < RS; ++i)
-#pragma unroll
-                for (int c = 0; c < NB; ++c) x[i][c] = pn[(tx + 32 * i) * PLD + c];
-            gj_panel_steps<B, RS, NB>(x, used, nb, k0, tx, perm, invk);
-#pragma unroll
-            for (int i = 0; i < RS; ++i)
-#pragma unroll
-                for (int c = 0; c < NB; ++c) fs[(tx + 32 * i) * PLD + c] = x[i][c];
-            __threadfence_block();
-            named_arrive(BAR_F, T);
-        }
-    } else {
-        // ---- update warps ----------------------------------------------------------------
-        float* yw = Yw + (size_t)w * NB * YL;
-#pragma unroll
-        for (int s = 0; s < SPW; ++s)
-#pragma unroll
-            for (int i = 0; i < RS; ++i) Pn[(tx + 32 * i) * PLD + w + W * s] = a[i][s];
-        __threadfence_block();
-        named_arrive(BAR_PANEL, T);
-#pragma unroll 1
-        for (int t = 0; t < NP; ++t) {
-            const int k0 = t * NB;
-            const int nb = (B - k0) < NB ? (B - k0) : NB;
-            const float* fs = Fs + (t & 1) * R32 * PLD;
-            named_sync(BAR_F, T);
-            // pivot rows of this warp's non-panel columns; their own entries are rebuilt from F.
-            // Warp 0 may meanwhile be recording panel t+1's pivots in invk: a row it records
-            // reads as -1 or as a step >= k0 + NB, outside this panel's range either way.
-            __syncwarp();
-            float mrow[RS];
-            gj_gather_pivot_rows<RS, CS, SPW, YL>(a, invk, k0, nb, tx, yw, mrow);
-            __syncwarp();
-            gj_clear_pivot_rows<RS, CS, SPW>(a, mrow);
-            // (1) slots SPW .. 2 SPW - 1 first: the next panel's columns, handed to warp 0 at once
-            // (at the last panel they hold earlier columns, updated like the rest)
-#pragma unroll
-            for (int s = 0; s < NB; ++s) {
-                if (s >= nb) break;   // uniform
-                float f[RS];
-#pragma unroll
-                for (int i = 0; i < RS; ++i) f[i] = fs[(tx + 32 * i) * PLD + s];
-                const float* yr = yw + s * YL;
-#pragma unroll
-                for (int q = 0; q < SPW; ++q) {
-                    const float yv = yr[q];
-#pragma unroll
-                    for (int i = 0; i < RS; ++i) a[i][SPW + q] = fmaf(f[i], yv, a[i][SPW + q]);
-                }
-            }
-            if (t + 1 < NP) {
-                float* pn = Pn + ((t + 1) & 1) * R32 * PLD;
-#pragma unroll
-                for (int q = 0; q < SPW; ++q)
-#pragma unroll
-                    for (int i = 0; i < RS; ++i) pn[(tx + 32 * i) * PLD + w + W * q] = a[i][SPW + q];
-                __threadfence_block();
-                named_arrive(BAR_PANEL, T);
-            }
-            // (2) the remaining columns (slots 2 SPW .. CS - 1)
-#pragma unroll
-            for (int s = 0; s < NB; ++s) {
-                if (s >= nb) break;   // uniform
-                float f[RS];
-#pragma unroll
-                for (int i = 0; i < RS; ++i) f[i] = fs[(tx + 32 * i) * PLD + s];
-                const float* yr = yw + s * YL;
-#pragma unroll
-                for (int j0 = 0; j0 < CS - SPW; j0 += 4) {
-                    const float4 y4 = *reinterpret_cast<const float4*>(yr + j0);
-                    const float yv[4] = {y4.x, y4.y, y4.z, y4.w};
-#pragma unroll
-                    for (int q = 0; q < 4; q += 2)
-                        gj_update_pair<RS, CS, 2 * SPW>(a, f, SPW + j0 + q, yv[q], yv[q + 1]);
-                }
-            }
-            // (3) the panel's own columns become F
-#pragma unroll
-            for (int s = 0; s < SPW; ++s)
-#pragma unroll
-                for (int i = 0; i < RS; ++i) a[i][s] = fs[(tx + 32 * i) * PLD + w + W * s];
-#pragma unroll
-            for (int i = 0; i < RS; ++i) {
-                float t0[SPW];
-#pragma unroll
-                for (int s = 0; s < SPW; ++s) t0[s] = a[i][s];
-#pragma unroll
-                for (int j = 0; j < CS - SPW; ++j) a[i][j] = a[i][j + SPW];
-#pragma unroll
-                for (int s = 0; s < SPW; ++s) a[i][CS - SPW + s] = t0[s];
-            }
-        }
-    }
-    __syncthreads();
-    if (wq > 0) {
-#pragma unroll
-        for (int i = 0; i < RS; ++i)
-#pragma unroll
-            for (int j = 0; j < CS; ++j) {
-                const int r = tx + 32 * i, c = w + W * j;
-                if (r < B && c < B) tile[perm[c] * LD + invk[r]] = a[i][j];
-            }
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < B * B; t += T) g[t] = tile[(t / B) * LD + (t % B)];
-}
-
 // ---- variants of the FP32 Gauss-Jordan kernel and their tuning --------------------------------
 // Two families.  Unblocked (variants 0..13): variant v < 4 unrolls the pivot loop kGjUnroll[v]
 // times (0 = fully, only for B <= 100); 4..8 are the column-owner form with kGjWarps[v - 4]
 // warps per element (valid while a thread's share of the block stays at most 128 values);
-// 9..13 the rotating column-owner form with kGjWarps[v - 9] warps.  Blocked (14..21):
-// k_gj_blk with kGjBlkWarps[v - 14] warps and the look-ahead k_gj_la with 1 + kGjBlkWarps[v - 18]
-// warps (valid while a thread holds at most 64 values).
+// 9..13 the rotating column-owner form with kGjWarps[v - 9] warps.  Blocked (14..17):
+// k_gj_blk with kGjBlkWarps[v - 14] warps (valid while a thread holds at most 64 values).  The split form
+// of 2-D levels is a family of its own.
 // Within a family the variants do the same arithmetic in the same order, so the tuner's choice
 // never changes a result; the tuner times one family only (the blocked one where it is valid,
 // unless emg_params.block_kernels asks for the unblocked forms).
@@ -598,8 +428,7 @@ constexpr int kGjUnroll[] = {1, 4, 16, 0};
 constexpr int kGjWarps[] = {1, 2, 4, 8, 16};
 constexpr int kGjBlkWarps[] = {1, 2, 4, 8};
 constexpr int kGjBlkFirst = 14;
-constexpr int kGjLaFirst = 18;   // look-ahead form, kGjBlkWarps[v - 18] update warps
-constexpr int kGjVariants = 22;
+constexpr int kGjVariants = 18;
 
 template <int B, int W>
 constexpr bool gj_blk_valid() {
@@ -610,14 +439,6 @@ template <int B>
 static bool gj_variant_valid(int v) {
     if (v < 0 || v >= kGjVariants) return false;
     if (v < 4) return kGjUnroll[v] != 0 || B <= 100;
-    if (v >= kGjLaFirst) {
-        switch (kGjBlkWarps[v - kGjLaFirst]) {
-            case 1: return GjLa<B, 1>::VALID;
-            case 2: return GjLa<B, 2>::VALID;
-            case 4: return GjLa<B, 4>::VALID;
-            default: return GjLa<B, 8>::VALID;
-        }
-    }
     if (v >= kGjBlkFirst) {
         switch (kGjBlkWarps[v - kGjBlkFirst]) {
             case 1: return gj_blk_valid<B, 1>();
@@ -632,7 +453,6 @@ static bool gj_variant_valid(int v) {
 
 static std::string gj_variant_name(int v) {
     if (v < 4) return "tile unroll " + std::to_string(kGjUnroll[v]);
-    if (v >= kGjLaFirst) return "look-ahead 1+" + std::to_string(kGjBlkWarps[v - kGjLaFirst]) + " warps";
     if (v >= kGjBlkFirst) return "blocked " + std::to_string(kGjBlkWarps[v - kGjBlkFirst]) + " warps";
     return std::string(v < 9 ? "cols " : "rotating cols ") + std::to_string(kGjWarps[(v - 4) % 5]) + " warps";
 }
@@ -644,19 +464,6 @@ static cudaError_t gj_blk_go(unsigned E, float* blk, cudaStream_t st) {
         cudaError_t e = cudaFuncSetAttribute(k_gj_blk<B, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
         k_gj_blk<B, W><<<E, 32 * W, sm, st>>>((int)E, blk, nullptr, nullptr);
-        return cudaGetLastError();
-    } else {
-        return cudaErrorInvalidValue;   // not reached: gj_dispatch checks the variant first
-    }
-}
-
-template <int B, int W>
-static cudaError_t gj_la_go(unsigned E, float* blk, cudaStream_t st) {
-    if constexpr (GjLa<B, W>::VALID) {
-        const size_t sm = GjLa<B, W>::SMEM;
-        cudaError_t e = cudaFuncSetAttribute(k_gj_la<B, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_gj_la<B, W><<<E, GjLa<B, W>::THREADS, sm, st>>>((int)E, blk);
         return cudaGetLastError();
     } else {
         return cudaErrorInvalidValue;   // not reached: gj_dispatch checks the variant first
@@ -712,10 +519,6 @@ static bool gj_split_ok(int B, int v) {
 template <int B>
 static cudaError_t gj_launch(int v, unsigned E, float* blk, cudaStream_t st) {
     switch (v) {
-        case 18: return gj_la_go<B, 1>(E, blk, st);
-        case 19: return gj_la_go<B, 2>(E, blk, st);
-        case 20: return gj_la_go<B, 4>(E, blk, st);
-        case 21: return gj_la_go<B, 8>(E, blk, st);
         case 14: return gj_blk_go<B, 1>(E, blk, st);
         case 15: return gj_blk_go<B, 2>(E, blk, st);
         case 16: return gj_blk_go<B, 4>(E, blk, st);
@@ -798,7 +601,7 @@ emg_status tune_gj(emg_ctx* c) {
         if (c->prm.block_kernels != 3)
             for (int v = kGjBlkFirst; v < kGjVariants; ++v) blocked = blocked || gj_valid(L.B, v);
         const int v_lo = blocked && !L.gj_split ? kGjBlkFirst : 0;
-        const int v_hi = L.gj_split ? 4 : blocked ? kGjVariants : kGjBlkFirst;   // 0..3 / 14..21 / 0..13
+        const int v_hi = L.gj_split ? 4 : blocked ? kGjVariants : kGjBlkFirst;   // 0..3 / 14..17 / 0..13
         auto valid = [&](int v) { return L.gj_split ? gj_split_ok(L.B, v) : gj_valid(L.B, v); };
         auto name = [&](int v) {
             return L.gj_split ? "split " + std::to_string(kGjBlkWarps[v]) + " warps" : gj_variant_name(v);
