@@ -92,6 +92,7 @@ struct LevelDev {
     double* fjr = nullptr;     // [F_int][QF][25] w|n dS| dF~/dU_R
     double* blk = nullptr;     // [E][B][B]      P_e, then its LU factors (column-major)
     int* piv = nullptr;        // [E][B] (float32 forms of 2-D levels: GjWork, blocks.cuh)
+    int* lu_list = nullptr;    // FP64 form, 2-D: [E + 2] blocks that do not split, their number, a ticket
     // FP32 block path (EMG_PREC_FP32_BLOCKS): float copies of the tables and blocks
     float* vpsi32 = nullptr;
     float* vgw32 = nullptr;

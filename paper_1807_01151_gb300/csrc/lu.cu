@@ -12,10 +12,10 @@
 //
 // A block whose spanwise momentum (variable 3) is coupled to no other variable, every entry of its
 // rows and columns outside the 3-3 block being exactly 0 (2-D flow in the plane), splits into
-// systems of 4 N and N unknowns.  k_lu finds that by looking at the block, factors the two apart
-// and marks it (kSplit in the first pivot); k_stage then solves the large one, and the small one
-// only where r has a spanwise part.  The operations left out all have a factor 0, so the factors and
-// solutions are those of the whole block.
+// systems of 4 N and N unknowns.  k_lu_split (2-D levels) finds that by looking at the block, factors the
+// two apart and marks it (kSplit in the first pivot), or puts it on a list for k_lu; k_stage then
+// solves the large one, and the small one only where r has a spanwise part.  The operations left out all
+// have a factor 0, so the factors and solutions are those of the whole block.
 #include <type_traits>
 
 #include "blocks.cuh"
@@ -38,6 +38,106 @@ __device__ __forceinline__ int seg_size(bool split, int seg) {
     return !split ? B : seg ? B / 5 : B / 5 * 4;
 }
 
+// Factorisation of an n x n system in shared memory (row stride LD) by 1 + WX WY warps, threads tid = 0
+// .. of the block; barriers under id 1, so that other warps of the block may do something else.
+// Bound by the float64 pipe (n^3 / 3 multiply-adds) and, per step, two barriers: warp 0 updates the
+// next column and finds its pivot while the other warps update the rest.  A warp's update tile is 8
+// rows by 4 columns (not 1 by 32), which wastes fewer lanes on the shrinking trailing block, and a
+// warp issues only the tiles it has: an operation whose lanes are all off takes the pipe as long (4560
+// float64 warp instructions a 60 x 60 block with four tiles always, 2900 needed).
+template <int n, int LD, int WX, int WY>
+__device__ __forceinline__ void lu_factor(double* a, int* rid, volatile int* s_piv, volatile double* s_inv, int tid) {
+    constexpr int T = 32 * (1 + WX * WY), GX = 4 * WX, GY = 8 * WY;
+    const int lane = tid & 31, w = (tid >> 5) - 1;
+    const int tx = (w % WX) * 4 + (lane & 3), ty = (w / WX) * 8 + (lane >> 2);
+    auto barrier = []() { asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory"); };
+    // warp 0: the pivot row of step t (the first of the largest |a|), its reciprocal, the row order
+    auto find_pivot = [&](int t) {
+        long long best = -2;   // every key is >= -1: a NaN row is taken only if no row is a number
+        int bi = t;
+        for (int r = t + lane; r < n; r += 32) {
+            const long long v = piv_key(a[r * LD + t]);
+            if (v > best) {
+                best = v;
+                bi = r;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ob > best || (ob == best && oi < bi)) {
+                best = ob;
+                bi = oi;
+            }
+        }
+        const double inv = rcp_h3(a[bi * LD + t]);
+        if (lane == 0) {
+            *s_piv = bi;
+            *s_inv = inv;
+            const int r0 = rid[t];
+            rid[t] = rid[bi];
+            rid[bi] = r0;
+        }
+    };
+    if (w < 0) find_pivot(0);
+    barrier();
+#pragma unroll 1
+    for (int t = 0; t < n; ++t) {
+        const int pr = *s_piv;
+        const double inv = *s_inv;
+        // swap rows t and pr outside column t; column t: the multipliers of the rows below, with the
+        // row that was t at pr, and the pivot's reciprocal
+        for (int c = tid; c < n; c += T) {
+            if (c != t && pr != t) {
+                const double t0 = a[t * LD + c];
+                a[t * LD + c] = a[pr * LD + c];
+                a[pr * LD + c] = t0;
+            }
+            if (c > t && c != pr) a[c * LD + t] *= inv;
+            if (c == t) {
+                if (pr != t) a[pr * LD + t] = a[t * LD + t] * inv;
+                a[t * LD + t] = inv;
+            }
+        }
+        barrier();
+        if (w < 0) {
+            // the next column first, then its pivot, while the other warps update the rest
+            if (t + 1 < n) {
+                const double u = a[t * LD + t + 1];
+                for (int r = t + 1 + lane; r < n; r += 32) a[r * LD + t + 1] = fma(-a[r * LD + t], u, a[r * LD + t + 1]);
+                __syncwarp();
+                find_pivot(t + 1);
+            }
+        } else {
+            // NP of the tiles c0 + p GX at a time, as many as the warp has
+            auto tiles = [&](auto np, int c0) {
+                constexpr int NP = decltype(np)::value;
+                double u[NP];
+#pragma unroll
+                for (int p = 0; p < NP; ++p) u[p] = c0 + p * GX < n ? a[t * LD + c0 + p * GX] : 0.0;
+                for (int r = t + 1 + ty; r < n; r += GY) {
+                    double* row = a + r * LD + c0;
+                    const double l = a[r * LD + t];
+#pragma unroll
+                    for (int p = 0; p < NP; ++p)
+                        if (c0 + p * GX < n) row[p * GX] = fma(-l, u[p], row[p * GX]);
+                }
+            };
+            for (int c0 = t + 2 + tx, cw = c0 - (lane & 3); cw < n; c0 += 4 * GX, cw += 4 * GX) {
+                if (cw + 3 * GX < n)
+                    tiles(std::integral_constant<int, 4>{}, c0);
+                else if (cw + 2 * GX < n)
+                    tiles(std::integral_constant<int, 3>{}, c0);
+                else if (cw + GX < n)
+                    tiles(std::integral_constant<int, 2>{}, c0);
+                else
+                    tiles(std::integral_constant<int, 1>{}, c0);
+            }
+        }
+        barrier();
+    }
+}
+
 template <int B>
 struct LuCfg {
     static constexpr int LD = (B + 3) / 8 * 8 + 4;   // row stride: 8 x 4 tiles of a warp hit every bank once
@@ -48,124 +148,128 @@ struct LuCfg {
     static_assert(LD >= B && LD % 8 == 4, "row stride");
 };
 
-// Bound by the float64 pipe (B^3 / 3 multiply-adds) and, per step, two barriers: warp 0 updates the
-// next column and finds its pivot while the other warps update the rest.  A warp's update tile is 8
-// rows by 4 columns (not 1 by 32), which wastes fewer lanes on the shrinking trailing block.  128 x 64 O-grid, FP64 V-cycle at p = 4: 9.5 ms with search, swap, scaling and a 1-by-32
-// update of the whole 75 x 75 block each behind a barrier, 8.0 ms as it is (the float64 pipe 73 %
-// busy, the division of a step a correctly rounded one: 8.3).
+// Every block of the level (list = nullptr, one CTA each), or those that k_lu_split left.
 template <int B>
-__global__ void __launch_bounds__(LuCfg<B>::THREADS) k_lu(int E, double* __restrict__ blk, int* __restrict__ piv) {
+__global__ void __launch_bounds__(LuCfg<B>::THREADS) k_lu(int E, double* __restrict__ blk, int* __restrict__ piv,
+                                                         const int* __restrict__ list, int* __restrict__ head) {
     using C = LuCfg<B>;
-    constexpr int LD = C::LD, T = C::THREADS, N = B / 5, GX = 4 * C::WX, GY = 8 * C::WY;
+    constexpr int LD = C::LD, T = C::THREADS;
     extern __shared__ __align__(16) unsigned char smraw[];
     double* a = reinterpret_cast<double*>(smraw);
     __shared__ int rid[B], s_piv;
     __shared__ double s_inv;
+    const int tid = threadIdx.x;
+    const int ne = list ? take_list(head) : E;
+#pragma unroll 1
+    for (int it = blockIdx.x; it < ne; it += gridDim.x) {
+        const int e = list ? list[it] : it;
+        double* g = blk + (size_t)e * B * B;
+        __syncthreads();
+        for (int t = tid; t < B * B; t += T) a[(t / B) * LD + t % B] = g[t];
+        for (int t = tid; t < B; t += T) rid[t] = t;
+        __syncthreads();
+        lu_factor<B, LD, C::WX, C::WY>(a, rid, &s_piv, &s_inv, tid);
+        __syncthreads();
+        for (int t = tid; t < B; t += T) piv[(size_t)e * B + t] = rid[t];
+        // column-major out: g[col * B + row]
+        for (int t = tid; t < B * B; t += T) g[t] = a[(t % B) * LD + t / B];
+    }
+}
+
+// 2-D levels: the 4 N x 4 N system by the first warps, the N x N one by the last warp beside them.
+// What is left out of shared memory lets six blocks share an SM at N = 15 (four with the whole block).
+// FP64 V-cycle of the 128 x 64 O-grid at p = 4: 8.0 -> 4.9 ms in factorisations, 19.4 -> 16.3 ms in all.
+template <int N>
+struct LuSplit {
+    static constexpr int B4 = 4 * N, LD = (B4 + 3) / 8 * 8 + 4, LD3 = N | 1;
+    static constexpr int WX = N <= 6 ? 2 : 4, WY = N <= 3 ? 1 : N <= 10 ? 1 : 2;
+    static constexpr int MAIN = 32 * (1 + WX * WY), THREADS = MAIN + 32;
+    static constexpr size_t SMEM = (size_t)(B4 * LD + N * LD3) * sizeof(double);
+    static constexpr int MINB = N == 15 ? 6 : N == 10 ? 10 : 16;
+};
+template <int N>
+__global__ void __launch_bounds__(LuSplit<N>::THREADS, LuSplit<N>::MINB) k_lu_split(int E, double* __restrict__ blk,
+                                                                                    int* __restrict__ piv,
+                                                                                    int* __restrict__ list,
+                                                                                    int* __restrict__ head) {
+    using C = LuSplit<N>;
+    constexpr int B = 5 * N, B4 = C::B4, LD = C::LD, LD3 = C::LD3, T = C::THREADS;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double* a = reinterpret_cast<double*>(smraw);
+    double* a3 = a + B4 * LD;
+    __shared__ int rid[B4], rid3[N], s_piv;
+    __shared__ double s_inv;
     const int e = blockIdx.x, tid = threadIdx.x;
     double* g = blk + (size_t)e * B * B;
     bool coupled = false;
+#pragma unroll 4
     for (int t = tid; t < B * B; t += T) {
-        const int r = t / B, c = t % B;
+        const int r = t / B, c = t - r * B, rs = r / N, cs = c / N;
         const double v = g[t];
-        a[r * LD + c] = v;
-        coupled |= (r / N == 3) != (c / N == 3) && !(v == 0.0);
+        if (rs != 3 && cs != 3)
+            a[(rs == 4 ? r - N : r) * LD + (cs == 4 ? c - N : c)] = v;
+        else if (rs == cs)
+            a3[(r - 3 * N) * LD3 + c - 3 * N] = v;
+        else
+            coupled |= !(v == 0.0);
     }
-    for (int t = tid; t < B; t += T) rid[t] = t;
-    const bool split = !__syncthreads_or(coupled);
-    const int lane = tid & 31, w = (tid >> 5) - 1;
-    const int tx = (w % C::WX) * 4 + (lane & 3), ty = (w / C::WX) * 8 + (lane >> 2);
+    for (int t = tid; t < B4; t += T) rid[t] = t;
+    if (__syncthreads_or(coupled)) {
+        if (tid == 0) list[atomicAdd(head, 1)] = e;
+        return;
+    }
+    if (tid < C::MAIN) {
+        lu_factor<B4, LD, C::WX, C::WY>(a, rid, &s_piv, &s_inv, tid);
+    } else {   // lane r: row r
+        const int lane = tid & 31;
+        if (lane < N) rid3[lane] = lane;
+        __syncwarp();
 #pragma unroll 1
-    for (int seg = 0; seg < (split ? 2 : 1); ++seg) {
-        const int n = seg_size<B>(split, seg);
-        // warp 0: the pivot row of step t (the first of the largest |a|), its reciprocal, the row order
-        auto find_pivot = [&](int t) {
-            const int k = seg_at<B>(split, seg, t);
-            long long best = -2;   // every key is >= -1: a NaN row is taken only if no row is a number
-            int bi = k;
-            for (int c = t + lane; c < n; c += 32) {
-                const int r = seg_at<B>(split, seg, c);
-                const long long v = piv_key(a[r * LD + k]);
-                if (v > best) {
-                    best = v;
-                    bi = r;
-                }
-            }
+        for (int t = 0; t < N; ++t) {
+            long long best = lane >= t && lane < N ? piv_key(a3[lane * LD3 + t]) : -2;
+            int p = lane >= t && lane < N ? lane : t;
             for (int o = 16; o > 0; o >>= 1) {
                 const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ob > best || (ob == best && oi < bi)) {
+                const int oi = __shfl_xor_sync(0xffffffffu, p, o);
+                if (ob > best || (ob == best && oi < p)) {
                     best = ob;
-                    bi = oi;
+                    p = oi;
                 }
             }
-            const double inv = rcp_h3(a[bi * LD + k]);
+            const double inv = rcp_h3(a3[p * LD3 + t]);
+            __syncwarp();
+            if (lane < N && p != t) {
+                const double t0 = a3[t * LD3 + lane];
+                a3[t * LD3 + lane] = a3[p * LD3 + lane];
+                a3[p * LD3 + lane] = t0;
+            }
             if (lane == 0) {
-                s_piv = bi;
-                s_inv = inv;
-                const int r0 = rid[k];
-                rid[k] = rid[bi];
-                rid[bi] = r0;
+                const int r0 = rid3[t];
+                rid3[t] = rid3[p];
+                rid3[p] = r0;
             }
-        };
-        if (w < 0) find_pivot(0);
-        __syncthreads();
-#pragma unroll 1
-        for (int t = 0; t < n; ++t) {
-            const int k = seg_at<B>(split, seg, t);
-            const int pr = s_piv;
-            const double inv = s_inv;
-            // swap rows k and pr outside column k; column k: the multipliers of the rows below, with the
-            // row that was k at pr, and the pivot's reciprocal
-            for (int c = tid; c < n; c += T) {
-                const int cc = seg_at<B>(split, seg, c);
-                if (c != t && pr != k) {
-                    const double t0 = a[k * LD + cc];
-                    a[k * LD + cc] = a[pr * LD + cc];
-                    a[pr * LD + cc] = t0;
-                }
-                if (c > t && cc != pr) a[cc * LD + k] *= inv;
-                if (c == t) {
-                    if (pr != k) a[pr * LD + k] = a[k * LD + k] * inv;
-                    a[k * LD + k] = inv;
-                }
+            __syncwarp();
+            if (lane > t && lane < N) {
+                const double l = a3[lane * LD3 + t] * inv;
+                a3[lane * LD3 + t] = l;
+                for (int c = t + 1; c < N; ++c) a3[lane * LD3 + c] = fma(-l, a3[t * LD3 + c], a3[lane * LD3 + c]);
             }
-            __syncthreads();
-            if (w < 0) {
-                // the next column first, then its pivot, while the other warps update the rest
-                if (t + 1 < n) {
-                    const int kn = seg_at<B>(split, seg, t + 1);
-                    const double u = a[k * LD + kn];
-                    for (int c = t + 1 + lane; c < n; c += 32) {
-                        double* row = a + seg_at<B>(split, seg, c) * LD;
-                        row[kn] = fma(-row[k], u, row[kn]);
-                    }
-                    __syncwarp();
-                    find_pivot(t + 1);
-                }
-            } else {
-                for (int c0 = t + 2 + tx; c0 < n; c0 += 4 * GX) {
-                    double u[4];
-                    int cc[4];
-#pragma unroll
-                    for (int p = 0; p < 4; ++p) {
-                        cc[p] = c0 + p * GX < n ? seg_at<B>(split, seg, c0 + p * GX) : -1;
-                        u[p] = cc[p] >= 0 ? a[k * LD + cc[p]] : 0.0;
-                    }
-                    for (int r = t + 1 + ty; r < n; r += GY) {
-                        double* row = a + seg_at<B>(split, seg, r) * LD;
-                        const double l = row[k];
-#pragma unroll
-                        for (int p = 0; p < 4; ++p)
-                            if (cc[p] >= 0) row[cc[p]] = fma(-l, u[p], row[cc[p]]);
-                    }
-                }
-            }
-            __syncthreads();
+            if (lane == t) a3[t * LD3 + t] = inv;
+            __syncwarp();
         }
     }
-    for (int t = tid; t < B; t += T) piv[(size_t)e * B + t] = rid[t] | (split && t == 0 ? kSplit : 0);
-    // column-major out: g[col * B + row]
-    for (int t = tid; t < B * B; t += T) g[t] = a[(t % B) * LD + t / B];
+    __syncthreads();
+    for (int t = tid; t < B; t += T) {
+        const int s = t / N;
+        const int r = s == 3 ? 3 * N + rid3[t - 3 * N] : rid[s == 4 ? t - N : t];
+        piv[(size_t)e * B + t] = (s != 3 && r >= 3 * N ? r + N : r) | (t == 0 ? kSplit : 0);
+    }
+    // column-major out: g[col * B + row], the two systems' places only
+    for (int t = tid; t < B4 * B4; t += T) {
+        const int c = t / B4, r = t % B4;
+        g[(size_t)seg_at<B>(true, 0, c) * B + seg_at<B>(true, 0, r)] = a[r * LD + c];
+    }
+    for (int t = tid; t < N * N; t += T) g[(size_t)(3 * N + t / N) * B + 3 * N + t % N] = a3[t % N * LD3 + t / N];
 }
 
 // The same factorisation for blocks that do not fit in shared memory (B = 175 in float64):
@@ -447,29 +551,38 @@ __global__ void __launch_bounds__(128) k_stage_gemv(int E, const float* __restri
     }
 }
 
-static emg_status lu_dispatch(emg_ctx* c, int B, double* blk, int* piv) {
+template <int N>
+static emg_status lu_split(emg_ctx* c, LevelDev& L) {
+    using C = LuSplit<N>;
+    EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_lu_split<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+    EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_lu<5 * N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LuCfg<5 * N>::SMEM));
     const unsigned E = (unsigned)c->E;
-    switch (B) {
-#define EMG_LU_CASE(BB)                                                                                      \
-    case BB: {                                                                                               \
-        if constexpr (LuCfg<BB>::SMEM > 227 * 1024) {                                                        \
-            ProfScope _ps(c, PC_LU);                                                                         \
-            k_lu_gmem<BB><<<E, 256, 0, c->stream>>>((int)E, blk, piv);                                       \
-        } else {                                                                                             \
-            const size_t sm = LuCfg<BB>::SMEM;                                                               \
-            EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_lu<BB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
-            ProfScope _ps(c, PC_LU);                                                                         \
-            k_lu<BB><<<E, LuCfg<BB>::THREADS, sm, c->stream>>>((int)E, blk, piv);                            \
-        }                                                                                                    \
-        EMG_CHECK_LAUNCH(c);                                                                                 \
-        return EMG_OK;                                                                                       \
+    {
+        ProfScope _ps(c, PC_LU);
+        k_lu_split<N><<<E, C::THREADS, C::SMEM, c->stream>>>((int)E, L.blk, L.piv, L.lu_list, L.lu_list + E);
     }
-        EMG_BSIZES(EMG_LU_CASE)
-#undef EMG_LU_CASE
-        default:
-            c->err = "unsupported block size";
-            return EMG_ERR_ARG;
+    EMG_CHECK_LAUNCH(c);
+    ProfScope _ps(c, PC_LU);
+    k_lu<5 * N><<<E < kListBlocks ? E : kListBlocks, LuCfg<5 * N>::THREADS, LuCfg<5 * N>::SMEM, c->stream>>>(
+        (int)E, L.blk, L.piv, L.lu_list, L.lu_list + E);
+    EMG_CHECK_LAUNCH(c);
+    return EMG_OK;
+}
+
+template <int B>
+static emg_status lu_whole(emg_ctx* c, LevelDev& L) {
+    const unsigned E = (unsigned)c->E;
+    if constexpr (LuCfg<B>::SMEM > 227 * 1024) {
+        ProfScope _ps(c, PC_LU);
+        k_lu_gmem<B><<<E, 256, 0, c->stream>>>((int)E, L.blk, L.piv);
+    } else {
+        const size_t sm = LuCfg<B>::SMEM;
+        EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_lu<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        ProfScope _ps(c, PC_LU);
+        k_lu<B><<<E, LuCfg<B>::THREADS, sm, c->stream>>>((int)E, L.blk, L.piv, nullptr, nullptr);
     }
+    EMG_CHECK_LAUNCH(c);
+    return EMG_OK;
 }
 
 static emg_status stage_dispatch(emg_ctx* c, int B, const double* lu, const int* piv, const double* r,
@@ -491,7 +604,21 @@ static emg_status stage_dispatch(emg_ctx* c, int B, const double* lu, const int*
     }
 }
 
-emg_status launch_lu(emg_ctx* c, int p) { return lu_dispatch(c, c->lv[p].B, c->lv[p].blk, c->lv[p].piv); }
+emg_status launch_lu(emg_ctx* c, int p) {
+    LevelDev& L = c->lv[p];
+    if (c->dim == 2) switch (p) {
+            case 1: return lu_split<3>(c, L);
+            case 2: return lu_split<6>(c, L);
+            case 3: return lu_split<10>(c, L);
+            default: return lu_split<15>(c, L);
+        }
+    switch (p) {
+        case 1: return lu_whole<20>(c, L);
+        case 2: return lu_whole<50>(c, L);
+        case 3: return lu_whole<100>(c, L);
+        default: return lu_whole<175>(c, L);
+    }
+}
 
 emg_status launch_stage(emg_ctx* c, int p, const double* r, const double* un, double beta, double* out) {
     LevelDev& L = c->lv[p];

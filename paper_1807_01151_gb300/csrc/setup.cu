@@ -434,7 +434,7 @@ int64_t estimate_bytes(int dim, int64_t E, int64_t F, int64_t F_int, int p_max, 
             if (blocks_f32(prec))
                 b += E * B * B * 4 + E * Q * N * (1 + dim) * 4 + F * QF * (N + 25) * 4 + Fi1 * QF * (N + 25) * 4;
             else
-                b += E * B * B * 8;
+                b += E * B * B * 8 + (dim == 2 ? (E + 2) * 4 : 0);
             b += E * B * 4;                                                     // pivots
         }
     }
@@ -625,6 +625,10 @@ emg_status setup_device_mesh(emg_ctx* c, const emg_mesh_desc* m) {
                 EMG_ALLOC(L.fjr32, float, std::max<int64_t>(F_int, 1) * L.QF * 25);
             } else {
                 EMG_ALLOC(L.blk, double, E * L.B * L.B);
+                if (D == 2) {
+                    EMG_ALLOC(L.lu_list, int, E + 2);
+                    EMG_CUDA_TRY(c, cudaMemsetAsync(L.lu_list, 0, (E + 2) * sizeof(int), c->stream));
+                }
             }
             EMG_ALLOC(L.piv, int, E * L.B);
         }
