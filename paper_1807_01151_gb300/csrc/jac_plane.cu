@@ -22,6 +22,9 @@ struct DiagPl {
     static constexpr int N = L::N, Q = L::Q, QF = L::QF, FP = 4 * QF, B4 = 4 * N;
     static constexpr int EC = 30 / N;                     // elements per block
     static constexpr int THREADS = 160;
+    // resident blocks: four would leave N = 15 96 registers a thread, 40 too few (340 bytes spilled; the
+    // smoothing step of 8192 elements at p = 4 1237 -> 1200 us with three, 18432 elements 2448 -> 2397)
+    static constexpr int MINB = N == 15 ? 3 : 4;
     static constexpr int NPAD = (N + 3) / 4 * 4;
     // shared memory (floats), per kind [EC][...]
     static constexpr int O_PS = 0;                        // [Q + FP][NPAD]   basis at the points
@@ -36,7 +39,7 @@ struct DiagPl {
 };
 
 template <int P>
-__global__ void __launch_bounds__(160, 4) k_diag_blocks_pl(
+__global__ void __launch_bounds__(160, DiagPl<P>::MINB) k_diag_blocks_pl(
     int E, int nmax, const double* __restrict__ u, const float* __restrict__ vpsi, const float* __restrict__ vgw,
     const int* __restrict__ elem_face, const float* __restrict__ fpsiL, const float* __restrict__ fpsiR,
     const float* __restrict__ fjl, const float* __restrict__ fjr, const double* __restrict__ psic,
