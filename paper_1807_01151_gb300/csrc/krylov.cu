@@ -38,39 +38,45 @@ __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned nblocks, unsign
     if (threadIdx.x == 0) {
         const unsigned target = (*epoch + 1u) * nblocks;
         *epoch += 1u;
-        __threadfence();
-        const unsigned arrived = atomicAdd(&bar->count, 1u) + 1u;
+        // release: this block's writes before the arrival; acquire: the others' before what follows
+        unsigned seen;
+        asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(seen) : "l"(&bar->count) : "memory");
         int ok = 1;
-        if (arrived < target) {
-            volatile unsigned int* vc = &bar->count;
-            const long long t0 = clock64();
-            while (*vc < target) {
-                if (clock64() - t0 > budget) {
-                    atomicExch(&sc->timeout, 1);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(20);
+        const long long t0 = clock64();
+        for (unsigned n = 1;; ++n) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&bar->count) : "memory");
+            if (seen >= target) break;
+            // another block that gave up never arrives: its flag is looked at now and then
+            if (clock64() - t0 > budget || (n % 64 == 0 && *((volatile int*)&sc->timeout))) {
+                atomicExch(&sc->timeout, 1);
+                ok = 0;
+                break;
             }
         }
-        __threadfence();
-        *s_ok = ok && !*((volatile int*)&sc->timeout);
+        *s_ok = ok;
     }
     __syncthreads();
     return *s_ok != 0;
 }
 
 constexpr int ARN_THREADS = 256;
-constexpr int ARN_PER_THREAD = 1;   // spread the FP64 work over every SM (FP64 is slow per SM)
 
-// Blocks of the persistent Arnoldi launch: about ARN_PER_THREAD entries per thread, at most
-// what is co-resident (per_sm per SM) and at most `cap`.
+// Blocks of the Arnoldi process, at most `cap` and what is co-resident (per_sm per SM; two, as the form with
+// rows in registers).  More blocks share out the rows' work, fewer make the cross-block reductions
+// shorter, which every block repeats.  Measured, us of an EXP1 step (m = 30) with 64, 128, 192 and 256 rows a
+// block: float64, whose pipe a block of 256 rows fills, 2560 rows 739 747 801 872, 10240 rows 887 756 806
+// 880, 23040 rows 1111 1132 840 905, 40960 rows 1319 (304 blocks) 1322 1352 1384; float32 2560 rows 478
+// 479 495 491, 10240 rows 511 487 496 490, 23040 rows 669 585 525 518, 40960 rows 717 720 664 619.
+template <class T>
 static int64_t arnoldi_blocks(int64_t K0, int nsm, int per_sm, int64_t cap) {
-    int64_t nb = (K0 + (int64_t)ARN_THREADS * ARN_PER_THREAD - 1) / ((int64_t)ARN_THREADS * ARN_PER_THREAD);
-    const int64_t resident = (int64_t)nsm * (per_sm < 1 ? 1 : per_sm);
-    if (nb > resident) nb = resident;
-    if (nb > cap) nb = cap;
-    return nb < 1 ? 1 : nb;
+    auto blocks = [K0](int64_t rows) { return (K0 + rows - 1) / rows; };
+    const int64_t resident = (int64_t)nsm * std::max(1, std::min(per_sm, 2));
+    int64_t nb;
+    if (sizeof(T) == 4)
+        nb = blocks(K0 <= 10240 ? 128 : 256);
+    else
+        nb = blocks(128) <= nsm ? blocks(128) : blocks(192) <= nsm ? blocks(192) : resident;
+    return std::max<int64_t>(1, std::min({nb, resident, cap}));
 }
 constexpr int ARN_CHUNK = 8;  // vectors per dot-product sweep
 static_assert(ARN_CHUNK == 8, "warp_sum8 reduces eight columns");
@@ -78,6 +84,7 @@ static_assert(ARN_CHUNK == 8, "warp_sum8 reduces eight columns");
 constexpr int ARN_MAXCOL = MAX_KRYLOV + 8;
 constexpr int ARN_WARPS = ARN_THREADS / 32;
 constexpr int ARN_SUB = 8;    // threads per column in the cross-block reduction
+constexpr int ARN_LOADS = 20;
 
 // Arithmetic of the Arnoldi process in the basis' precision T (double, or float for the float32
 // Krylov form): explicit fused multiply-adds (so that every form of the process computes the
@@ -145,8 +152,8 @@ __device__ __forceinline__ void block_reduce_store(T v[ARN_CHUNK], int n, T* dst
 }
 
 // out_sh[c] = sum over blocks b of part[b * stride + c], c < ncol, identical in every block:
-// ARN_SUB threads per column sum a fixed stride of blocks (eight loads issued together, then
-// added in order), then a fixed shuffle tree.
+// ARN_SUB threads per column sum a fixed stride of blocks (ARN_LOADS loads issued together, then
+// added in order: one trip to L2 for 160 blocks), then a fixed shuffle tree.
 template <class T>
 __device__ __forceinline__ void reduce_cols(const T* part, int nb, int stride, int ncol, T* out_sh,
                                             T (*sh)[ARN_MAXCOL]) {
@@ -155,15 +162,15 @@ __device__ __forceinline__ void reduce_cols(const T* part, int nb, int stride, i
         const int c = c0 + threadIdx.x / ARN_SUB;
         T v = 0.0;
         if (c < ncol) {
-            for (int b0 = sub; b0 < nb; b0 += 8 * ARN_SUB) {
-                T x[8];
+            for (int b0 = sub; b0 < nb; b0 += ARN_LOADS * ARN_SUB) {
+                T x[ARN_LOADS];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                for (int u = 0; u < ARN_LOADS; ++u) {
                     const int b = b0 + u * ARN_SUB;
                     x[u] = b < nb ? __ldcg(part + (size_t)b * stride + c) : 0.0;   // other blocks' data: L2
                 }
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v += x[u];
+                for (int u = 0; u < ARN_LOADS; ++u) v += x[u];
             }
         }
         for (int o = ARN_SUB / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, ARN_SUB);
@@ -172,14 +179,17 @@ __device__ __forceinline__ void reduce_cols(const T* part, int nb, int stride, i
     __syncthreads();
 }
 
+// Warps of a block with n rows that have any: the others leave the pipes to them.
+__device__ __forceinline__ int arn_warps(int64_t n) { return n >= ARN_THREADS ? ARN_WARPS : n > 0 ? (int)((n + 31) / 32) : 0; }
+
 // dst[i] (i < nv) = V[i] . w over this block's slice, plus w . w at index nv if with_ww
 // (warp shuffles per chunk of columns, one barrier for all of them).
 template <class T>
 __device__ __forceinline__ void slice_dots(const T* V, const T* w, int64_t K0, int64_t k0, int64_t k1,
                                            int nv, int with_ww, T* dst, T (*sh)[ARN_MAXCOL]) {
     const int ncol = nv + with_ww;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int c0 = 0; c0 < ncol; c0 += ARN_CHUNK) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = arn_warps(k1 - k0);
+    for (int c0 = 0; c0 < ncol && warp < nw; c0 += ARN_CHUNK) {
         T v[ARN_CHUNK];
 #pragma unroll
         for (int i = 0; i < ARN_CHUNK; ++i) v[i] = 0.0;
@@ -199,7 +209,7 @@ __device__ __forceinline__ void slice_dots(const T* V, const T* w, int64_t K0, i
     __syncthreads();
     for (int c = threadIdx.x; c < ncol; c += ARN_THREADS) {
         T s = 0.0;
-        for (int wv = 0; wv < ARN_WARPS; ++wv) s += sh[wv][c];
+        for (int wv = 0; wv < nw; ++wv) s += sh[wv][c];
         dst[c] = s;
     }
 }
@@ -292,6 +302,28 @@ __device__ __forceinline__ void arn_half1(int j, int64_t K0, int64_t k0, int64_t
 // process continues (the same in every block).  Hs is the block's shared copy of H (row
 // stride ARN_HLD), complete up to column j - 1 on entry.
 constexpr int ARN_HLD = 41;   // row stride of the shared Hessenberg copy (m <= 40)
+// Sum of v[i]^2, i < n, the same in every thread: lanes, then a fixed shuffle tree (in a serial loop
+// every warp would take the float64 pipe n times).
+template <class T>
+__device__ __forceinline__ T arn_sum_sq(const T* v, int n) {
+    T s = 0.0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) s = fma_t(v[i], v[i], s);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+// c = H~_j h2 over l = 0..j+1, ARN_SUB threads per row.
+template <class T>
+__device__ __forceinline__ void arn_cs(int j, const T* Hs, const T* h2, T* cs) {
+    const int sub = threadIdx.x % ARN_SUB;
+    for (int l0 = 0; l0 <= j + 1; l0 += ARN_THREADS / ARN_SUB) {
+        const int l = l0 + threadIdx.x / ARN_SUB;
+        T c = 0.0;
+        if (l <= j + 1)
+            for (int i = (l > 0 ? l - 1 : 0) + sub; i <= j; i += ARN_SUB) c = fma_t(Hs[l * ARN_HLD + i], h2[i], c);
+        for (int o = ARN_SUB / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o, ARN_SUB);
+        if (sub == 0 && l <= j + 1) cs[l] = c;
+    }
+}
 template <class T>
 __device__ __forceinline__ bool arn_half2(int j, int m, int64_t K0, int64_t k0, int64_t k1, int nb, int stride,
                                           int NF, const double* __restrict__ bsr, const int* __restrict__ nbr,
@@ -300,8 +332,7 @@ __device__ __forceinline__ bool arn_half2(int j, int m, int64_t K0, int64_t k0, 
                                           const T* h1, T* h2, T* cs, DevScalars* sc,
                                           T (*sh)[ARN_MAXCOL]) {
     reduce_cols<T>(partB, nb, stride, j + 2, h2, sh);
-    T hh = 0.0;
-    for (int i = 0; i <= j; ++i) hh = fma_t(h2[i], h2[i], hh);
+    const T hh = arn_sum_sq<T>(h2, j + 1);
     const T hn = sqrt(fmax(h2[j + 1] - hh, (T)0));
     const T w0 = sqrt(h1[j + 1]);
     const bool brk = !(hn > arn_breakdown_tol<T>() * w0);
@@ -318,12 +349,7 @@ __device__ __forceinline__ bool arn_half2(int j, int m, int64_t K0, int64_t k0, 
     for (int i = threadIdx.x; i <= j + 1; i += ARN_THREADS) Hs[i * ARN_HLD + j] = i <= j ? h1[i] + h2[i] : hn;
     __syncthreads();
     const T ih = (T)1 / hn;
-    // c = H~_j h2 over l = 0..j+1
-    for (int l = threadIdx.x; l <= j + 1; l += ARN_THREADS) {
-        T c = 0.0;
-        for (int i = (l > 0 ? l - 1 : 0); i <= j; ++i) c = fma_t(Hs[l * ARN_HLD + i], h2[i], c);
-        cs[l] = c;
-    }
+    arn_cs<T>(j, Hs, h2, cs);
     __syncthreads();
     T* vn = V + (size_t)(j + 1) * K0;
     for (int64_t k = k0 + threadIdx.x; k < k1; k += ARN_THREADS) {
@@ -353,13 +379,13 @@ __device__ __forceinline__ bool arn_half2(int j, int m, int64_t K0, int64_t k0, 
 // barrier-free kernels', which share that form).  Loops over i <= j run over the register
 // array with a uniform early exit, so every index is a compile-time one.
 template <class T, int MV>
-__device__ __forceinline__ void slice_dots_rv(const T (&vrow)[MV], T wk, bool has, int nv, T* dst,
+__device__ __forceinline__ void slice_dots_rv(const T (&vrow)[MV], T wk, bool has, int nw, int nv, T* dst,
                                               T (*sh)[ARN_MAXCOL]) {
     const int ncol = nv + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
     for (int c0 = 0; c0 < MV + 1; c0 += ARN_CHUNK) {
-        if (c0 >= ncol) break;   // uniform
+        if (c0 >= ncol || warp >= nw) break;   // uniform over the warp
         T v[ARN_CHUNK];
 #pragma unroll
         for (int i = 0; i < ARN_CHUNK; ++i) v[i] = 0.0;
@@ -380,13 +406,13 @@ __device__ __forceinline__ void slice_dots_rv(const T (&vrow)[MV], T wk, bool ha
     __syncthreads();
     for (int c = threadIdx.x; c < ncol; c += ARN_THREADS) {
         T s = 0.0;
-        for (int wv = 0; wv < ARN_WARPS; ++wv) s += sh[wv][c];
+        for (int wv = 0; wv < nw; ++wv) s += sh[wv][c];
         dst[c] = s;
     }
 }
 
 template <class T, int MV>
-__device__ __forceinline__ void arn_half1_rv(int j, int nb, int stride, const T (&vrow)[MV], bool has, int64_t k,
+__device__ __forceinline__ void arn_half1_rv(int j, int nb, int stride, const T (&vrow)[MV], bool has, int nw, int64_t k,
                                              T* w, T& wk, const T* partA, T* partB_blk,
                                              T* h1, T (*sh)[ARN_MAXCOL]) {
     reduce_cols<T>(partA, nb, stride, j + 2, h1, sh);
@@ -402,19 +428,18 @@ __device__ __forceinline__ void arn_half1_rv(int j, int nb, int stride, const T 
     }
     wk = s;
     __syncthreads();
-    slice_dots_rv<T, MV>(vrow, s, has, j + 1, partB_blk, sh);
+    slice_dots_rv<T, MV>(vrow, s, has, nw, j + 1, partB_blk, sh);
 }
 
 template <class T, int MV>
-__device__ __forceinline__ bool arn_half2_rv(int j, int m, int64_t K0, int64_t k, bool has, int nb, int stride,
+__device__ __forceinline__ bool arn_half2_rv(int j, int m, int64_t K0, int64_t k, bool has, int nw, int nb, int stride,
                                              int NF, const double* __restrict__ bsr, const int* __restrict__ nbr,
                                              const double* __restrict__ dt, T* V, T (&vrow)[MV], T w1k,
                                              const T* w1, T* wn, double* H, T* Hs, const T* partB,
                                              T* partA_blk, const T* h1, T* h2, T* cs,
                                              DevScalars* sc, T (*sh)[ARN_MAXCOL]) {
     reduce_cols<T>(partB, nb, stride, j + 2, h2, sh);
-    T hh = 0.0;
-    for (int i = 0; i <= j; ++i) hh = fma_t(h2[i], h2[i], hh);
+    const T hh = arn_sum_sq<T>(h2, j + 1);
     const T hn = sqrt(fmax(h2[j + 1] - hh, (T)0));
     const T w0 = sqrt(h1[j + 1]);
     const bool brk = !(hn > arn_breakdown_tol<T>() * w0);
@@ -431,11 +456,7 @@ __device__ __forceinline__ bool arn_half2_rv(int j, int m, int64_t K0, int64_t k
     for (int i = threadIdx.x; i <= j + 1; i += ARN_THREADS) Hs[i * ARN_HLD + j] = i <= j ? h1[i] + h2[i] : hn;
     __syncthreads();
     const T ih = (T)1 / hn;
-    for (int l = threadIdx.x; l <= j + 1; l += ARN_THREADS) {
-        T c = 0.0;
-        for (int i = (l > 0 ? l - 1 : 0); i <= j; ++i) c = fma_t(Hs[l * ARN_HLD + i], h2[i], c);
-        cs[l] = c;
-    }
+    arn_cs<T>(j, Hs, h2, cs);
     __syncthreads();
     T wnk = 0.0;
     if (has) {
@@ -458,7 +479,7 @@ __device__ __forceinline__ bool arn_half2_rv(int j, int m, int64_t K0, int64_t k
         wn[k] = wnk;
     }
     __syncthreads();
-    slice_dots_rv<T, MV>(vrow, wnk, has, j + 2, partA_blk, sh);
+    slice_dots_rv<T, MV>(vrow, wnk, has, nw, j + 2, partA_blk, sh);
     return true;
 }
 
@@ -483,6 +504,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 2) k_arnoldi_rv(int64_t K0, int E
     const int64_t k1 = (k0 + chunk) < K0 ? (k0 + chunk) : K0;
     const int64_t k = k0 + threadIdx.x;
     const bool has = k < k1;
+    const int nw = arn_warps(k1 - k0);
     T vrow[MV];
 #pragma unroll
     for (int i = 0; i < MV; ++i) vrow[i] = 0.0;
@@ -511,14 +533,14 @@ __global__ void __launch_bounds__(ARN_THREADS, 2) k_arnoldi_rv(int64_t K0, int E
     }
     spmv_rows<T>(k0, k1, NF, bsr, nbr, dt, nullptr, r, ib, wbuf);   // A v_1 from the inputs: no barrier
     __syncthreads();
-    slice_dots_rv<T, MV>(vrow, has ? wbuf[k] : 0.0, has, 1, partA + (size_t)blockIdx.x * stride, sh);
+    slice_dots_rv<T, MV>(vrow, has ? wbuf[k] : 0.0, has, nw, 1, partA + (size_t)blockIdx.x * stride, sh);
     for (int j = 0; j < m; ++j) {
         T* w = wbuf + (size_t)(j & 1) * K0;
         if (!grid_sync(bar, nb, &epoch, budget, sc, &s_ok)) return;
         T w1k = 0.0;
-        arn_half1_rv<T, MV>(j, (int)nb, stride, vrow, has, k, w, w1k, partA, partB + (size_t)blockIdx.x * stride, h1, sh);
+        arn_half1_rv<T, MV>(j, (int)nb, stride, vrow, has, nw, k, w, w1k, partA, partB + (size_t)blockIdx.x * stride, h1, sh);
         if (!grid_sync(bar, nb, &epoch, budget, sc, &s_ok)) return;
-        if (!arn_half2_rv<T, MV>(j, m, K0, k, has, (int)nb, stride, NF, bsr, nbr, dt, V, vrow, w1k, w,
+        if (!arn_half2_rv<T, MV>(j, m, K0, k, has, nw, (int)nb, stride, NF, bsr, nbr, dt, V, vrow, w1k, w,
                               wbuf + (size_t)((j + 1) & 1) * K0, H, Hs, partB, partA + (size_t)blockIdx.x * stride, h1,
                               h2, cs, sc, sh))
             break;
@@ -1035,7 +1057,7 @@ static emg_status exp1_krylov(emg_ctx* c, const double* u0, const double* dt, do
     EMG_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_arnoldi<T>, ARN_THREADS, 0));
     EMG_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_rv, k_arnoldi_rv<T, ARN_RV>, ARN_THREADS, 0));
     EMG_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    const int64_t nb = arnoldi_blocks(K0, nsm, per_sm, c->red_blocks);
+    const int64_t nb = arnoldi_blocks<T>(K0, nsm, per_sm, c->red_blocks);
     // rows in registers: one row per thread at most, every block co-resident, m <= ARN_RV
     const bool rows_in_regs = m <= ARN_RV && (K0 + nb - 1) / nb <= ARN_THREADS && nb <= (int64_t)nsm * per_sm_rv;
     const int stride = MAX_KRYLOV + 8;
@@ -1222,7 +1244,7 @@ extern "C" emg_status emg_exp1_step_noalloc(int32_t dim, int64_t n_elems, const 
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_arnoldi<double>, ARN_THREADS, 0) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return EMG_ERR_CUDA;
-    const int64_t nb = arnoldi_blocks(K0, nsm, per_sm, NA_BLOCKS);
+    const int64_t nb = arnoldi_blocks<double>(K0, nsm, per_sm, NA_BLOCKS);
     int64_t K0a = K0;
     int Ea = (int)E, NFa = NF, ma = krylov_m, stra = NA_STRIDE;
     const double* bsrc = bsr;
