@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(TrCfg<D, P>::THREADS) k_traces(int E, const do
                                                                  const int2* __restrict__ fpsiR,
                                                                  const int2* __restrict__ texp,
                                                                  double* __restrict__ tr) {
+    chain_wait();
     using L = Lv<D, P>;
     using CF = TrCfg<D, P>;
     constexpr int N = L::N, QF = L::QF, B = L::B, NF = L::NF, NP = CF::NP, NS = CF::NS;
@@ -258,6 +259,7 @@ __global__ void __launch_bounds__(FaceCfg<D, P>::THREADS) k_face_flux(int F, int
                                                    double g, U5 uinf, FarField ff,
                                                    const double* __restrict__ fvr, double* __restrict__ fhat,
                                                    int* __restrict__ fkey) {
+    chain_wait();
     using CF = FaceCfg<D, P>;
     constexpr int QF = CF::QF, FB = CF::FB;
     __shared__ int mx[FB * 5];
@@ -488,6 +490,7 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
     const int2* __restrict__ texp, const int4* __restrict__ fhat, const int* __restrict__ fkey,
     const double* __restrict__ tau, double g,
     const double* __restrict__ vvr, U5 om, double* __restrict__ R) {
+    chain_wait();
     using L = Lv<D, P>;
     using CF = VolCfg<D, P, S>;
     using GT = GradTab<D, P>;
@@ -696,6 +699,7 @@ __global__ void __launch_bounds__(128) k_cell0(int E, const double* __restrict__
                                                const double* __restrict__ fpsiL, const double* __restrict__ fpsiR,
                                                const double* __restrict__ fhat, const double* __restrict__ tau, U5 om,
                                                double* __restrict__ R) {
+    chain_wait();
     using L = Lv<D, 0>;
     constexpr int QF = L::QF, NF = L::NF;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -805,7 +809,7 @@ emg_status launch_traces(emg_ctx* c, int p, const double* u, double* tr, int cls
         using CF = TrCfg<DD, PP>;                                                                               \
         EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_traces<DD, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CF::SMEM)); \
         ProfScope _ps(c, cls);                                                                                  \
-        k_traces<DD, PP><<<(unsigned)((E + CF::ET - 1) / CF::ET), CF::THREADS, CF::SMEM, c->stream>>>(          \
+        launch_chained(c, k_traces<DD, PP>, (unsigned)((E + CF::ET - 1) / CF::ET), CF::THREADS, CF::SMEM, \
             E, u, c->elem_face, reinterpret_cast<const int2*>(L.fpsiL), reinterpret_cast<const int2*>(L.fpsiR), \
             L.texp, tr);                                                                                        \
     }
@@ -815,10 +819,14 @@ emg_status launch_traces(emg_ctx* c, int p, const double* u, double* tr, int cls
     return EMG_OK;
 }
 
-// Below this many elements (about 13 per SM) the projections take four threads per mode: measured
-// 32 x 16 p = 1: 53.3 -> 28.7 us, the 32 x 16 p = 2 V-cycle 2.48 -> 2.22 ms; at 3234 hexes p = 4 the
-// four-thread form takes 948 us against 670.
-constexpr int VOL_SMALL_ELEMS = 2000;
+// Below this many elements the projections take four threads per mode.  Where the line lies, measured per
+// residual (one thread / four threads a mode), us: 2-D p = 1 8192 elements 55.5 / 50.5, 18432 82.2 / 82.9;
+// p = 2 4608 45.4 / 45.6, 8192 59.7 / 72.1; p = 3 1152 38.2 / 34.1, 2048 45.3 / 47.9; p = 4 1152 39.2 / 37.1,
+// 2048 48.1 / 51.5; 3-D p = 1 4608 103 / 80, 13824 209 / 212; p = 2 2352 130 / 109, 4608 184 / 200; p = 3
+// 216 95 / 63, 900 143 / 145; p = 4 216 135 / 111, 900 226 / 272.
+constexpr int vol_small_elems(int D, int P) {
+    return D == 2 ? (P == 1 ? 16000 : P == 2 ? 4500 : 1500) : P == 1 ? 10000 : P == 2 ? 3500 : P == 3 ? 800 : 450;
+}
 
 emg_status launch_residual(emg_ctx* c, int p, const double* u, const double* tau, double* R) {
     LevelDev& L = c->lv[p];
@@ -842,19 +850,19 @@ emg_status launch_residual(emg_ctx* c, int p, const double* u, const double* tau
 #define EMG_RES_ROT(DD, PP, RR)                                                                                 \
     {                                                                                                          \
         using FC = FaceCfg<DD, PP>;                                                                            \
-        { ProfScope _ps(c, PC_RES_FACE); k_face_flux<DD, PP, RR><<<(unsigned)((F + FC::FB - 1) / FC::FB), FC::THREADS, 0, c->stream>>>( \
+        { ProfScope _ps(c, PC_RES_FACE); launch_chained(c, k_face_flux<DD, PP, RR>, (unsigned)((F + FC::FB - 1) / FC::FB), FC::THREADS, 0, \
             F, Fi, c->face_L, c->face_R, c->face_bc, L.fnrm, L.famag, L.fpsiL, L.fpsiR, L.fwn, u, L.tr, g, ui, ff,     \
             L.fvr, L.fhat, L.fkey); }                                                                                         \
         EMG_CHECK_LAUNCH(c);                                                                                   \
         ProfScope _ps(c, PC_RES_VOL);                                                                          \
         if constexpr (PP == 0) {                                                                               \
-            k_cell0<DD, RR><<<(unsigned)((E + 127) / 128), 128, 0, c->stream>>>(E, u, c->elem_face, L.fpsiL,   \
+            launch_chained(c, k_cell0<DD, RR>, (unsigned)((E + 127) / 128), 128, 0, E, u, c->elem_face, L.fpsiL,   \
                 L.fpsiR, L.fhat, tau, om, R);                                                                  \
         } else {                                                                                               \
-            const bool small = E < VOL_SMALL_ELEMS;                                                            \
+            const bool small = E < vol_small_elems(DD, PP);                                                            \
             const int ET = small ? VolCfg<DD, PP, true>::ET : VolCfg<DD, PP, false>::ET;                       \
             const int T = small ? VolCfg<DD, PP, true>::THREADS : VolCfg<DD, PP, false>::THREADS;              \
-            (small ? k_volume<DD, PP, RR, true> : k_volume<DD, PP, RR, false>)<<<(unsigned)((E + ET - 1) / ET), T, 0, c->stream>>>( \
+            launch_chained(c, (small ? k_volume<DD, PP, RR, true> : k_volume<DD, PP, RR, false>), (unsigned)((E + ET - 1) / ET), T, 0, \
                 E, u, reinterpret_cast<const int2*>(L.vpsi), reinterpret_cast<const int2*>(L.vgw),             \
                 c->elem_face, reinterpret_cast<const int2*>(L.fpsiL), reinterpret_cast<const int2*>(L.fpsiR),  \
                 L.texp, reinterpret_cast<const int4*>(L.fhat), L.fkey, tau, g, L.vvr, om, R);                                                         \
