@@ -146,7 +146,7 @@ typedef struct {
                               1: the tensor-core forms (tcgen05: 3xTF32 assembly, blocked
                               Gauss-Jordan with rank-16 MMA updates for B = 75, 100, 175);
                               2: the SIMT (FMA) forms (blocked Gauss-Jordan with rank-8
-                              updates where a thread's share fits 64 registers, else the
+                              updates where a thread's share fits its registers, else the
                               unblocked column-owner form); 3: the SIMT forms with the
                               unblocked Gauss-Jordan everywhere.  The forms differ only in
                               rounding; the BF16 form always assembles on the tensor cores. */

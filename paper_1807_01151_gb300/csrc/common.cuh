@@ -35,10 +35,7 @@ inline bool use_tc_assembly(int dim, int p, int prec, int block_kernels) {
     return false;
 }
 inline bool use_tc_inverse(int B, int block_kernels) {
-    const bool built = B == 75 || B == 100 || B == 175;
-    if (!built || block_kernels >= 2) return false;
-    if (block_kernels == 1) return true;
-    return false;
+    return block_kernels == 1 && (B == 75 || B == 100 || B == 175);
 }
 
 __host__ __device__ constexpr int n_modes(int D, int P) {

@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(LuCfg<B>::THREADS) k_lu(int E, double* __restr
 
 // 2-D levels: the 4 N x 4 N system by the first warps, the N x N one by the last warp beside them.
 // What is left out of shared memory lets six blocks share an SM at N = 15 (four with the whole block).
-// FP64 V-cycle of the 128 x 64 O-grid at p = 4: 8.0 -> 4.9 ms in factorisations, 19.4 -> 16.3 ms in all.
+// FP64 V-cycle of the 128 x 64 O-grid at p = 4: 8.0 -> 4.75 ms in factorisations, 19.5 -> 16.3 ms in all.
 template <int N>
 struct LuSplit {
     static constexpr int B4 = 4 * N, LD = (B4 + 3) / 8 * 8 + 4, LD3 = N | 1;
