@@ -127,4 +127,11 @@ __device__ __forceinline__ double rsqrt_h3(double a) {
     return fma(e * y, fma(0.375, e, 0.5), y);
 }
 
+// b / a, negative if either number is: its square root is then NaN as sqrt(a) or sqrt(b) would be, also
+// where both are negative (a state without a meaning must not look like one with).
+__device__ __forceinline__ double ratio_or_negative(double b, double ia, double a) {
+    const double r = b * ia;
+    return __hiloint2double(__double2hiint(r) | (__double2hiint(a) & (int)0x80000000), __double2loint(r));
+}
+
 }  // namespace emg

@@ -49,7 +49,7 @@ struct RoeV {
 template <int NK>
 __device__ __forceinline__ void roe_of(const SideV<NK>& L, const SideV<NK>& R, const double n[3], double g, double vrn,
                                        RoeV<NK>& w) {
-    const double s2 = R.r * L.ir, s = s2 * rsqrt_h3(s2);
+    const double s2 = ratio_or_negative(R.r, L.ir, L.r), s = s2 * rsqrt_h3(s2);
     w.wR = s * rcp_h3(1.0 + s);
     w.rho = s * L.r;
     w.K = 0.0;

@@ -156,7 +156,7 @@ __device__ __forceinline__ void roe_flux_fast(const double UL[5], const double U
     const double pL = (g - 1.0) * fma(-0.5, kL, UL[4]), pR = (g - 1.0) * fma(-0.5, kR, UR[4]);
     const double EL = UL[4] + pL, ER = UR[4] + pR;
     const double HL = EL * irL, HR = ER * irR;
-    const double s2 = UR[0] * irL;
+    const double s2 = ratio_or_negative(UR[0], irL, UL[0]);
     const double s = s2 * rsqrt_h3(s2);                 // sqrt(rho_R / rho_L)
     const double wR = s * rcp_h3(1.0 + s);              // s_R / (s_L + s_R)
     const double rho = s * UL[0];
