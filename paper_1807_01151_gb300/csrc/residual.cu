@@ -134,8 +134,10 @@ __global__ void __launch_bounds__(TrCfg<D, P>::THREADS) k_traces(int E, const do
 // ---- face fluxes ---------------------------------------------------------------------------------
 // The Roe flux of euler.cuh's roe_flux in float64, scaled by am, with four special functions
 // instead of seven: one reciprocal for both densities, sqrt(rho_R / rho_L) for the averages (weights
-// 1 / (1 + s) and s / (1 + s)), and one reciprocal square root for c and 1 / c^2.  NK = 2: a face in
-// the x-y plane between states without a z momentum (every z term is 0).
+// 1 / (1 + s) and s / (1 + s)), and one reciprocal square root for c and 1 / c^2.  The jumps are
+// differences of rounded numbers (not fused with the product before them), so that equal states have
+// none: the flux along a wall or through a uniform flow is free of dissipation to the last bit.  NK = 2:
+// a face in the x-y plane between states without a z momentum (every z term is 0).
 template <int NK, bool ROT>
 __device__ __forceinline__ void roe_flux_fast(const double UL[5], const double UR[5], const double n[3], double g,
                                               double vrn, double am, double F[5]) {
@@ -151,7 +153,7 @@ __device__ __forceinline__ void roe_flux_fast(const double UL[5], const double U
         kR = fma(UR[1 + k], vR, kR);
         qL = fma(vL[k], n[k], qL);
         qR = fma(vR, n[k], qR);
-        dv[k] = vR - vL[k];
+        dv[k] = __dsub_rn(vR, vL[k]);
     }
     const double pL = (g - 1.0) * fma(-0.5, kL, UL[4]), pR = (g - 1.0) * fma(-0.5, kR, UR[4]);
     const double EL = UL[4] + pL, ER = UR[4] + pR;
@@ -172,7 +174,7 @@ __device__ __forceinline__ void roe_flux_fast(const double UL[5], const double U
     const double c = c2 * ic, ic2 = ic * ic;
     const double dqn = qR - qL;
     const double qn = fma(wR, dqn, qL);
-    const double drho = UR[0] - UL[0], dp = pR - pL;
+    const double drho = UR[0] - UL[0], dp = __dsub_rn(pR, pL);
     const double rq = rho * c * dqn, hc = 0.5 * ic2;
     const double qr = ROT ? qn - vrn : qn;
     const double l2 = fabs(qr);
