@@ -65,7 +65,8 @@ struct LevelDev {
     // (p >= 1: fixed point, fix.cuh, two 32-bit halves in the place of each float64; p = 0: float64)
     double* vpsi = nullptr;    // [E][N][Q]      psi_i(x_q)
     double* vgw = nullptr;     // [E][D][Q][N]   W_q d_k psi_i(x_q)  (fixed point: rows q D + k, GradTab)
-    int2* texp = nullptr;      // [E]            their exponents: of psi (volume and face points), of vgw
+    int* texp = nullptr;       // [E]            exponent of psi (volume and face points)
+    int* gexp = nullptr;       // [E][D][N]      exponents of vgw, one for each direction and mode
     double* fnrm = nullptr;    // [F][QF][3]     unit outward normal of the L element
     double* famag = nullptr;   // [F][QF]        w |n dS|
     double* fpsiL = nullptr;   // [F][QF][N]     psi^L_i at the face points  (fixed point: FaceTab)

@@ -76,7 +76,7 @@ template <int D, int P>
 __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_diag_blocks_fx(
     int E, int nmax, const double* __restrict__ u, const int2* __restrict__ vpsi, const int2* __restrict__ vgw,
     const int* __restrict__ elem_face, const int2* __restrict__ fpsiL, const int2* __restrict__ fpsiR,
-    const int2* __restrict__ texp, const double* __restrict__ fjl, const double* __restrict__ fjr,
+    const int* __restrict__ texp, const int* __restrict__ gexp, const double* __restrict__ fjl, const double* __restrict__ fjr,
     const double* __restrict__ psic, const double* __restrict__ hlen, const double* __restrict__ cfl_dev, double g,
     int shifted, const double* __restrict__ vvr, double* __restrict__ out) {
     using C = DiagFx<D, P>;
@@ -92,10 +92,14 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
     __shared__ double ud[B], Us[Q][5], s_dtau;
     __shared__ int mxa[25], mxj[25], sa[25], sj[25], live[25], nlive;
     const int e = blockIdx.x, tid = threadIdx.x;
-    const int2 te = texp[e];
+    // the element's exponents of the basis values and, the least of its modes and directions, the gradients
+    __shared__ int ge[D * N];
+    for (int t = tid; t < D * N; t += T) ge[t] = gexp[(size_t)e * D * N + t];
     for (int t = tid; t < B; t += T) ud[t] = u[(size_t)e * B + t];
     if (tid < 25) mxa[tid] = mxj[tid] = 0;
+    int2 te = make_int2(texp[e], 0x7fffffff);
     __syncthreads();
+    for (int t = 0; t < D * N; ++t) te.y = min(te.y, ge[t]);
     // U at the volume points (float64: 5 N multiply-adds a point), dtau of Eq. x3d
     {
         const double sp = fix_scale(-te.x, 0);
@@ -172,7 +176,7 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
         const int2* gv = vgw + (size_t)e * D * Q * N;
         for (int t = tid; t < nq * D * N; t += T) {
             const int r = t / N, i = t % N;
-            gs[t] = gv[GradTab<D, P>::at(q0 * D + r, i)];
+            gs[t] = fix_shift(gv[GradTab<D, P>::at(q0 * D + r, i)], ge[r % D * N + i] - te.y, false);
         }
         if (Q == QC) {
             for (int t = tid; t < Q * D * 25; t += T) As[t] = fix_of(Ad[t], sa[t % 25]);
@@ -333,7 +337,7 @@ emg_status launch_diag_blocks_fx(emg_ctx* c, int p, const double* u, const doubl
         ProfScope _ps(c, PC_DIAG);                                                                                 \
         k_diag_blocks_fx<DD, PP><<<(unsigned)c->E, C::THREADS, C::SMEM, c->stream>>>(                              \
             (int)c->E, nmax, u, reinterpret_cast<const int2*>(L.vpsi), reinterpret_cast<const int2*>(L.vgw),       \
-            c->elem_face, reinterpret_cast<const int2*>(L.fpsiL), reinterpret_cast<const int2*>(L.fpsiR), L.texp,  \
+            c->elem_face, reinterpret_cast<const int2*>(L.fpsiL), reinterpret_cast<const int2*>(L.fpsiR), L.texp, L.gexp, \
             L.fjl, L.fjr, c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, out);                              \
     }
     EMG_DISPATCH_DP(c->dim, p, EMG_FX)

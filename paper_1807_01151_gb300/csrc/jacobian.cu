@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
     const int* __restrict__ elem_face, const T* __restrict__ fpsiL, const T* __restrict__ fpsiR,
     const T* __restrict__ fjl, const T* __restrict__ fjr, const double* __restrict__ psic,
     const double* __restrict__ hlen, const double* __restrict__ cfl_dev, double g, int shifted,
-    const double* __restrict__ vvr, const int2* __restrict__ texp, T* __restrict__ out) {
+    const double* __restrict__ vvr, const int* __restrict__ texp, const int* __restrict__ gexp, T* __restrict__ out) {
     using L = Lv<D, P>;
     constexpr int N = L::N, Q = L::Q, QF = L::QF, B = L::B, NF = L::NF;
     constexpr int QC = DiagCfg<D, P>::QC;
@@ -122,11 +122,8 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
         const double cs = sqrt(g * pr * ir);
         s_dtau = cfl_dev[0] * hlen[e] / ((2 * P + 1) * (sqrt(q2) + cs));
     }
-    double s_psi = 1.0, s_gw = 1.0;
-    if constexpr (FX) {
-        const int2 te = texp[e];
-        s_psi = fix_scale(-te.x, 0), s_gw = fix_scale(-te.y, 0);
-    }
+    double s_psi = 1.0;
+    if constexpr (FX) s_psi = fix_scale(-texp[e], 0);
     const bool active = tid < 25 * N;
     const int ab = tid / N, i = tid % N;
     const int a = ab / 5, b = ab % 5;
@@ -156,7 +153,8 @@ __global__ void __launch_bounds__(DiagCfg<D, P>::THREADS, (DiagMinB<D, P, T>::V)
                 const int k = t / (nq * N), r = t % (nq * N);
                 if constexpr (FX)
                     gs[r / N][k][r % N] = fix_back(reinterpret_cast<const int2*>(
-                        vgw)[(size_t)e * D * Q * N + GradTab<D, P>::at((q0 + r / N) * D + k, r % N)]) * s_gw;
+                        vgw)[(size_t)e * D * Q * N + GradTab<D, P>::at((q0 + r / N) * D + k, r % N)]) *
+                        fix_scale(-gexp[((size_t)e * D + k) * N + r % N], 0);
                 else
                     gs[r / N][k][r % N] = vgw[(((size_t)e * D + k) * Q + q0) * N + r];
             }
@@ -576,7 +574,7 @@ emg_status launch_diag_blocks(emg_ctx* c, int p, const double* u, const double* 
         ProfScope _ps(c, PC_DIAG);                                                                          \
         k_diag_blocks<DD, PP, double><<<(unsigned)c->E, DiagCfg<DD, PP>::THREADS, 0, c->stream>>>(          \
             (int)c->E, nmax, u, L.vpsi, L.vgw, c->elem_face, L.fpsiL, L.fpsiR, L.fjl, L.fjr, c->psic, c->h, \
-            cfl_dev, c->prm.gamma, shifted, L.vvr, L.texp, out);                                            \
+            cfl_dev, c->prm.gamma, shifted, L.vvr, L.texp, L.gexp, out);                                    \
     }
     EMG_DISPATCH_DP(c->dim, p, EMG_DB)
 #undef EMG_DB
@@ -612,7 +610,7 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
         if (c->prm.block_kernels == 3)                                                                      \
             k_diag_blocks<DD, PP, float><<<(unsigned)c->E, DiagCfg<DD, PP>::THREADS, 0, c->stream>>>(       \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
-                c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, nullptr, out);                        \
+                c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, nullptr, nullptr, out);               \
         else                                                                                                \
             k_diag_blocks_rb<DD, PP><<<grid, DiagRb<DD, PP>::THREADS, DiagRb<DD, PP>::SM * 4, c->stream>>>( \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \

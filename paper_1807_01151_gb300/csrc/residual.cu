@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(TrCfg<D, P>::THREADS) k_traces(int E, const do
                                                                  const int* __restrict__ elem_face,
                                                                  const int2* __restrict__ fpsiL,
                                                                  const int2* __restrict__ fpsiR,
-                                                                 const int2* __restrict__ texp,
+                                                                 const int* __restrict__ texp,
                                                                  double* __restrict__ tr) {
     chain_wait();
     using L = Lv<D, P>;
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(TrCfg<D, P>::THREADS) k_traces(int E, const do
     const int el = threadIdx.x / NP, pt = threadIdx.x % NP, e = e0 + el;
     if (el >= ET || e >= E) return;
     const int code = codes[el * NF + pt / QF];
-    const int st = texp[e].x;
+    const int st = texp[e];
     const int2* pr = ps + (size_t)threadIdx.x * NS;
     const int4* ur = reinterpret_cast<const int4*>(us + el * N * 6);
     long long h[5] = {0, 0, 0, 0, 0}, c[5] = {0, 0, 0, 0, 0};
@@ -352,8 +352,9 @@ __global__ void __launch_bounds__(FaceCfg<D, P>::THREADS) k_face_flux(int F, int
 // A block holds ET elements.  Points: thread (element, point) reconstructs U_h and its flux;
 // projections: thread (element, mode i) accumulates the five variables of R_{e,a,i}.  The fluxes
 // are staged in shared memory, first as float64, then in place as fixed point once the largest of
-// each (element, variable) is known: QC volume points at a time (all of them in 2-D), then the
-// faces', FC faces at a time as k_face_flux left them.
+// each (element, direction, variable) is known: QC volume points at a time (all of them in 2-D), then
+// the faces', FC faces at a time as k_face_flux left them.  Each direction has accumulators of its
+// own, so that its gradients and fluxes keep exponents of their own (fix.cuh).
 // S = false: a thread per mode, several elements a block (most work in flight per instruction
 // issued).  S = true, for meshes that leave the chip short of warps: four threads per mode, each
 // with a quarter of the rows, and fewer elements a block, so that each warp's chain of instructions
@@ -366,26 +367,30 @@ struct VolCfg {
     static constexpr int THREADS = S ? (TM <= 64 ? 64 : (TM + 31) / 32 * 32) : (D == 2 || L::N == 20) ? 64 : 128;
     static constexpr int ET = THREADS / TM;                          // elements per block
     static constexpr int FS = 6;                                     // padded variable stride
-    static constexpr int QMAX = FIX_TERMS / D;                       // points of one exact sum
+    static constexpr int QMAX = 54;                                  // points of one exact sum (more: no faster)
     static constexpr int QS = THREADS * 288 / (ET * D * FS * 8);     // points that fit the buffer
     static constexpr int QC0 = (QS < QMAX ? QS : QMAX) & ~1;
     static constexpr int QC = QC0 < L::Q ? QC0 : L::Q;               // points per chunk
     static constexpr int FC0 = (QC * D) / L::QF;                     // faces that fit the same buffer
-    static constexpr int FC = FC0 < 1 ? 1 : (FC0 > L::NF ? L::NF : FC0);
+    static constexpr int FC1 = FC0 < FIX_TERMS / L::QF ? FC0 : FIX_TERMS / L::QF;
+    static constexpr int FC = FC1 < 1 ? 1 : (FC1 > L::NF ? L::NF : FC1);
+    // the directions' sums are added with SH bits less: D QC 2^(56 - SH) < 2^63
+    static constexpr int SH = D * QC > 252 ? 2 : D * QC > 120 ? 1 : 0;
     static constexpr int ROWS = QC * D > FC * L::QF ? QC * D : FC * L::QF;
     static constexpr int MINB = 512 / THREADS;                       // 128 registers a thread
-    static constexpr int STAGES = (L::Q + QC - 1) / QC;
-    static_assert(QC >= 2 && FC * L::QF <= FIX_TERMS && QC * D <= FIX_TERMS && L::N <= FIX_TERMS, "exact sums");
+    static constexpr int KB = QC < L::Q ? 2 : 1;                     // buffers of the stages' keys
+    static_assert(QC >= 2 && FC * L::QF <= FIX_TERMS && QC <= FIX_TERMS && D * QC <= 504 && L::N <= FIX_TERMS, "exact sums");
 };
 
-// Largest keys of the rows that the warp's lanes add, one atomic per element and variable.
-__device__ __forceinline__ void row_max(int* mx, int el, const int key[5]) {
+// Largest of the keys that the warp's lanes hold for their elements, one atomic per element and key.
+template <int K>
+__device__ __forceinline__ void row_max(int* mx, int el, const int key[K]) {
     const unsigned grp = __match_any_sync(__activemask(), el);
     const bool lead = (threadIdx.x & 31) == __ffs(grp) - 1;
 #pragma unroll
-    for (int a = 0; a < 5; ++a) {
+    for (int a = 0; a < K; ++a) {
         const int m = __reduce_max_sync(grp, key[a]);
-        if (lead && m > 0) atomicMax(&mx[el * 5 + a], m);
+        if (lead && m > 0) atomicMax(&mx[el * K + a], m);
     }
 }
 
@@ -412,7 +417,7 @@ __device__ __forceinline__ void row_put(double* row, const double v[5]) {
 
 // One table entry p times the five variables of a row (W: with the spanwise momentum).
 template <bool W>
-__device__ __forceinline__ void row_mac(long long h[5], long long c[5], int2 p, const int4* r) {
+__device__ __forceinline__ void row_mac(long long* h, long long* c, int2 p, const int4* r) {
     const int4 a = r[0], b = r[1];
     const int2 d = reinterpret_cast<const int2*>(r)[4];
     fix_mac(h[0], c[0], p, make_int2(a.x, a.y));
@@ -424,14 +429,18 @@ __device__ __forceinline__ void row_mac(long long h[5], long long c[5], int2 p, 
 
 // h, c += sum over a thread's share of `rows` rows of table entry (row, mode) times the row; tab:
 // the thread's first entry of the row range (paired: mode i at 2 i); of PARTS threads, thread
-// `part` takes every PARTS-th pair.  The G loads of a group are issued ahead of its sums, the next
-// group's during them.  R: the number of rows where it is known at compile time, else 0.
-template <bool W, int N, bool PAIRED, int PARTS, int R>
-__device__ __forceinline__ void rows_mac(long long h[5], long long c[5], const int2* __restrict__ tab,
+// `part` takes every PARTS-th pair.  Row t goes to the sums of direction t % ND (ND = 3: a thread takes
+// three pairs, two points, at a time, so that a row's direction is known when compiling).  The G loads
+// of a group are issued ahead of its sums, the next group's during them.  R: the number of rows where
+// it is known at compile time, else 0.
+template <bool W, int ND, int N, bool PAIRED, int PARTS, int R>
+__device__ __forceinline__ void rows_mac(long long (&h)[ND * 5], long long (&c)[ND * 5], const int2* __restrict__ tab,
                                          const double* row, int rows, int part) {
+    static_assert(ND == 1 || PAIRED, "directions only in paired tables");
     const int4* r = reinterpret_cast<const int4*>(row);
     constexpr int K = R / 2 / PARTS;   // pairs of a thread, when they are the same for all
-    constexpr bool EVEN = PAIRED && R > 0 && R % (2 * PARTS) == 0;
+    constexpr bool EVEN = PAIRED && R > 0 && R % (2 * PARTS) == 0 && ND < 3;
+    constexpr int S = ND == 2 ? 5 : 0;   // the second row of a pair
     constexpr int G = !EVEN ? 4 : K % 4 == 0 ? 4 : K % 5 == 0 ? 5 : K % 3 == 0 ? 3 : K % 2 == 0 ? 2 : 1;
     if constexpr (EVEN) {
         const int4* t4 = reinterpret_cast<const int4*>(tab) + part * N;
@@ -447,14 +456,37 @@ __device__ __forceinline__ void rows_mac(long long h[5], long long c[5], const i
 #pragma unroll
             for (int g = 0; g < G; ++g) {
                 row_mac<W>(h, c, make_int2(p[g].x, p[g].y), r + (m0 + g) * PARTS * 6);
-                row_mac<W>(h, c, make_int2(p[g].z, p[g].w), r + (m0 + g) * PARTS * 6 + 3);
+                row_mac<W>(h + S, c + S, make_int2(p[g].z, p[g].w), r + (m0 + g) * PARTS * 6 + 3);
                 p[g] = nx[g];
             }
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             row_mac<W>(h, c, make_int2(p[g].x, p[g].y), r + (K - G + g) * PARTS * 6);
-            row_mac<W>(h, c, make_int2(p[g].z, p[g].w), r + (K - G + g) * PARTS * 6 + 3);
+            row_mac<W>(h + S, c + S, make_int2(p[g].z, p[g].w), r + (K - G + g) * PARTS * 6 + 3);
+        }
+    } else if constexpr (ND == 3) {
+        const int pairs = rows >> 1;
+        const int4* t4 = reinterpret_cast<const int4*>(tab);
+        int4 p[3];
+#pragma unroll
+        for (int g = 0; g < 3; ++g)
+            if (3 * part + g < pairs) p[g] = t4[(3 * part + g) * N];
+#pragma unroll 1
+        for (int m0 = 3 * part; m0 < pairs; m0 += 3 * PARTS) {
+            int4 nx[3];
+#pragma unroll
+            for (int g = 0; g < 3; ++g)
+                if (m0 + 3 * PARTS + g < pairs) nx[g] = t4[(m0 + 3 * PARTS + g) * N];
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+                const int m = m0 + g;
+                if (m < pairs) {
+                    row_mac<W>(h + 2 * g % 3 * 5, c + 2 * g % 3 * 5, make_int2(p[g].x, p[g].y), r + m * 6);
+                    row_mac<W>(h + (2 * g + 1) % 3 * 5, c + (2 * g + 1) % 3 * 5, make_int2(p[g].z, p[g].w), r + m * 6 + 3);
+                }
+                p[g] = nx[g];
+            }
         }
     } else if constexpr (PAIRED) {
         const int pairs = rows >> 1;
@@ -474,7 +506,7 @@ __device__ __forceinline__ void rows_mac(long long h[5], long long c[5], const i
                 const int m = m0 + g * PARTS;
                 if (m < pairs) {
                     row_mac<W>(h, c, make_int2(p[g].x, p[g].y), r + m * 6);
-                    row_mac<W>(h, c, make_int2(p[g].z, p[g].w), r + m * 6 + 3);
+                    row_mac<W>(h + S, c + S, make_int2(p[g].z, p[g].w), r + m * 6 + 3);
                 }
                 p[g] = nx[g];
             }
@@ -489,8 +521,8 @@ template <int D, int P, bool ROT, bool S>
 __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MINB) k_volume(
     int E, const double* __restrict__ u, const int2* __restrict__ vpsi, const int2* __restrict__ vgw,
     const int* __restrict__ elem_face, const int2* __restrict__ fpsiL, const int2* __restrict__ fpsiR,
-    const int2* __restrict__ texp, const int4* __restrict__ fhat, const int* __restrict__ fkey,
-    const double* __restrict__ tau, double g,
+    const int* __restrict__ texp, const int* __restrict__ gexp, const int4* __restrict__ fhat,
+    const int* __restrict__ fkey, const double* __restrict__ tau, double g,
     const double* __restrict__ vvr, U5 om, double* __restrict__ R) {
     chain_wait();
     using L = Lv<D, P>;
@@ -503,13 +535,13 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
     constexpr int RV = Q == QC ? Q * D : 0;   // rows of the volume term when it is one chunk
     __shared__ __align__(16) int2 us[ET * N * FS];          // [ET][N][6] coefficients
     __shared__ __align__(16) double Fs[ET * ROWS * FS];     // [ET][rows][6] staged fluxes
-    __shared__ int mxu[ET * 5], mx[CF::STAGES][ET * 5];     // largest keys, of each stage
+    __shared__ int mxu[ET * 5], mx[CF::KB][ET * D * 5];   // largest keys, of a stage and the next
     __shared__ int codes[ET * NF];
     const int e0 = blockIdx.x * ET;
-    for (int t = threadIdx.x; t < ET * 5; t += T) {
-        mxu[t] = 0;
+    for (int t = threadIdx.x; t < ET * D * 5; t += T) {
+        if (t < ET * 5) mxu[t] = 0;
 #pragma unroll
-        for (int s = 0; s < CF::STAGES; ++s) mx[s][t] = 0;
+        for (int s = 0; s < CF::KB; ++s) mx[s][t] = 0;
     }
     for (int t = threadIdx.x; t < ET * NF; t += T)
         codes[t] = e0 + t / NF < E ? elem_face[(size_t)e0 * NF + t] : 0;
@@ -537,27 +569,23 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
     const int el2 = threadIdx.x / CF::TM, i2 = threadIdx.x % CF::TM / PARTS, part = threadIdx.x % PARTS;
     const int e2 = e0 + el2;
     const bool own = el2 < ET && e2 < E;
-    const int2 te = own ? texp[e2] : make_int2(0, 0);
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    int stage = 0;
+    int stage = 0;   // which of the keys' buffers
     // exact sums to acc: the scale is 2^(56 - s_table - s_flux), NaN for a non-finite flux
-    const unsigned live = PARTS > 1 ? __ballot_sync(0xffffffffu, own) : 0u;
-    auto add_sums = [&](long long h[5], long long c[5], int st, const int* keys) {
+    auto add_sums = [&](const long long* h, const long long* c, int st, const int* keys, bool w) {
 #pragma unroll
         for (int a = 0; a < 5; ++a) {
-#pragma unroll
-            for (int o = 1; o < PARTS; o <<= 1) {
-                h[a] += __shfl_xor_sync(live, h[a], o);
-                c[a] += __shfl_xor_sync(live, c[a], o);
-            }
+            if (a == 3 && !w) continue;
             const int key = keys[a];
             acc[a] += fix_sum(h[a], c[a], fix_scale(FIX_BITS - st - fix_exp(key), key));
         }
     };
 #pragma unroll 1
-    for (int q0 = 0; q0 < Q; q0 += QC, ++stage) {
+    for (int q0 = 0; q0 < Q; q0 += QC, stage ^= CF::KB - 1) {
         const int nq = (Q - q0) < QC ? (Q - q0) : QC;
         __syncthreads();   // us staged / previous chunk consumed
+        if (q0 > 0)
+            for (int t = threadIdx.x; t < ET * D * 5; t += T) mx[stage ^ 1][t] = 0;   // for the next one
         // (1) U_h and the Euler flux at the chunk's points
         for (int t = threadIdx.x; t < ET * nq; t += T) {
             const int el = t / nq, qq = t % nq, e = e0 + el;
@@ -573,7 +601,7 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
 #pragma unroll 5
                 for (int i = 0; i < N; ++i) row_mac<false>(h, c, pr[i * Q], ur + i * 3);
             }
-            const int st = texp[e].x;
+            const int st = texp[e];
             double U[5];
 #pragma unroll
             for (int a = 0; a < 5; ++a) {
@@ -593,7 +621,7 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
             const double pr_ = (g - 1.0) * fma(-0.5, ke, U[4]);
             const double H = U[4] + pr_;
             const double vv[3] = {v0, v1, v2};
-            int key[5] = {0, 0, 0, 0, 0};
+            int key[D * 5];
 #pragma unroll
             for (int k = 0; k < D; ++k) {
                 double Fk[5];
@@ -607,30 +635,54 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
                     for (int a = 0; a < 5; ++a) Fk[a] = fma(-vr[k], U[a], Fk[a]);
                 }
 #pragma unroll
-                for (int a = 0; a < 5; ++a) key[a] = max(key[a], fix_key(Fk[a]));
+                for (int a = 0; a < 5; ++a) key[k * 5 + a] = fix_key(Fk[a]);
                 row_put(Fs + ((size_t)el * nq * D + qq * D + k) * FS, Fk);
             }
-            row_max(mx[stage], el, key);
+            row_max<D * 5>(mx[stage], el, key);
         }
         __syncthreads();
         for (int t = threadIdx.x; t < ne * D * nq; t += T)
-            row_fix<D>(Fs + (size_t)t * FS, mx[stage] + t / (D * nq) * 5);
+            row_fix<D>(Fs + (size_t)t * FS, mx[stage] + (t / (D * nq) * D + t % D) * 5);
         __syncthreads();
         // (2) projection on the gradients: sum_q sum_k W_q d_k psi_i F_k,a
         if (own) {
-            long long h[5] = {0, 0, 0, 0, 0}, c[5] = {0, 0, 0, 0, 0};
-            const int2* tab = vgw + (size_t)e2 * D * Q * N + (size_t)q0 * D * N + (GT::paired ? 2 * i2 : i2);
+            long long h[D * 5], c[D * 5];
+#pragma unroll
+            for (int a = 0; a < D * 5; ++a) h[a] = c[a] = 0;
+            const int2* tab = vgw + (size_t)e2 * D * Q * N + (size_t)q0 * D * N + 2 * i2;
             const double* row = Fs + (size_t)el2 * nq * D * FS;
-            int rows = nq * D;
-            if (D == 3 || mx[stage][el2 * 5 + 3] != 0)
-                rows_mac<true, N, GT::paired, PARTS, RV>(h, c, tab, row, rows, part);
+            const int* keys = mx[stage] + el2 * D * 5;
+            int rows = nq * D, ge[D];
+#pragma unroll
+            for (int k = 0; k < D; ++k) ge[k] = gexp[((size_t)e2 * D + k) * N + i2];
+            const bool w = D == 3 || (keys[3] | keys[8]) != 0;
+            if (w)
+                rows_mac<true, D, N, GT::paired, PARTS, RV>(h, c, tab, row, rows, part);
             else
-                rows_mac<false, N, GT::paired, PARTS, RV>(h, c, tab, row, rows, part);
-            if (GT::paired && (rows & 1) && part == 0) {   // the last row of an odd number
+                rows_mac<false, D, N, GT::paired, PARTS, RV>(h, c, tab, row, rows, part);
+            if (D == 3 && (rows & 1) && part == 0) {   // the last row of an odd number: direction 2
                 --rows;
-                row_mac<true>(h, c, (tab - i2)[(size_t)rows * N], reinterpret_cast<const int4*>(row) + rows * 3);
+                row_mac<true>(h + (D - 1) * 5, c + (D - 1) * 5, (tab - i2)[(size_t)rows * N],
+                              reinterpret_cast<const int4*>(row) + rows * 3);
             }
-            add_sums(h, c, te.y, mx[stage] + el2 * 5);
+            // the directions' sums at the largest one's exponent, then one conversion a variable (the
+            // float64 pipe's): the cut is 2^-56 of (largest gradient) (largest flux) of that direction
+#pragma unroll
+            for (int a = 0; a < 5; ++a) {
+                if (a == 3 && !w) continue;
+                int ek[D], lo = 0x7fffffff, key = 0;
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    ek[k] = ge[k] + fix_exp(keys[k * 5 + a]);
+                    lo = min(lo, ek[k]);
+                    key = max(key, keys[k * 5 + a]);
+                }
+                long long s = 0;
+#pragma unroll
+                for (int k = 0; k < D; ++k)
+                    s += (h[k * 5 + a] + ((c[k * 5 + a] + (1ll << (FIX_LO - 1))) >> FIX_LO)) >> min(ek[k] - lo + CF::SH, 63);
+                acc[a] += __ll2double_rn(s) * fix_scale(FIX_BITS + CF::SH - lo, key);
+            }
         }
     }
     // (3) faces: -(L side) / +(R side) sum_t psi_i(x_t) w|n dS| F~_a.  A row is shifted from its
@@ -672,13 +724,22 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
                 const int2* tab = side + (FT::paired ? 2 * i2 : i2);
                 const double* row = Fs + (size_t)(el2 * nf + lf) * QF * FS;
                 if (w)
-                    rows_mac<true, N, FT::paired, PARTS, QF>(h, c, tab, row, QF, part);
+                    rows_mac<true, 1, N, FT::paired, PARTS, QF>(h, c, tab, row, QF, part);
                 else
-                    rows_mac<false, N, FT::paired, PARTS, QF>(h, c, tab, row, QF, part);
+                    rows_mac<false, 1, N, FT::paired, PARTS, QF>(h, c, tab, row, QF, part);
                 if (FT::paired && (QF & 1) && part == 0)
                     row_mac<true>(h, c, side[(QF - 1) * N + i2], reinterpret_cast<const int4*>(row) + (QF - 1) * 3);
             }
-            add_sums(h, c, te.x, mxu + el2 * 5);
+            add_sums(h, c, texp[e2], mxu + el2 * 5, w);
+        }
+    }
+    if constexpr (PARTS > 1) {   // the parts' sums of a mode, on neighbouring lanes
+        const unsigned live = __ballot_sync(0xffffffffu, own);
+        if (own) {
+#pragma unroll
+            for (int a = 0; a < 5; ++a)
+#pragma unroll
+                for (int o = 1; o < PARTS; o <<= 1) acc[a] += __shfl_xor_sync(live, acc[a], o);
         }
     }
     if (!own || part != 0) return;
@@ -733,45 +794,47 @@ __global__ void __launch_bounds__(128) k_cell0(int E, const double* __restrict__
 }
 
 // ---- fixed-point tables (set-up) --------------------------------------------------------------------
-// One block per element: the exponents of its basis values (volume and own face points) and
-// weighted gradients, then its tables in place as fixed point and in the residual's layouts: vpsi
+// One block per element: the exponents of its basis values (volume and own face points) and of its
+// weighted gradients of each direction and mode, then its tables in place as fixed point and in the residual's layouts: vpsi
 // from [Q][N] to [N][Q] (k_volume's threads, one per point, read it side by side), vgw from
 // [D][Q][N] and the face sides from [QF][N] to row pairs.
 template <int D, int P>
 __global__ void __launch_bounds__(128) k_fix_tables(double* __restrict__ vpsi, double* __restrict__ vgw,
                                                     const int* __restrict__ elem_face, double* __restrict__ fpsiL,
-                                                    double* __restrict__ fpsiR, int2* __restrict__ texp) {
+                                                    double* __restrict__ fpsiR, int* __restrict__ texp,
+                                                    int* __restrict__ gexp) {
     using L = Lv<D, P>;
     constexpr int N = L::N, Q = L::Q, QF = L::QF, NF = L::NF;
     extern __shared__ __align__(16) double buf[];   // [D][Q][N] at most
-    __shared__ int mx[2];
+    __shared__ int mx, mxg[D * N];
     const int e = blockIdx.x, tid = threadIdx.x;
     double* vp = vpsi + (size_t)e * Q * N;
     double* vg = vgw + (size_t)e * D * Q * N;
-    if (tid < 2) mx[tid] = 0;
+    if (tid == 0) mx = 0;
+    for (int t = tid; t < D * N; t += 128) mxg[t] = 0;
     __syncthreads();
-    int a = 0, b = 0;
+    int a = 0;
     for (int t = tid; t < Q * N; t += 128) a = max(a, fix_key(vp[t]));
-    for (int t = tid; t < D * Q * N; t += 128) b = max(b, fix_key(vg[t]));
+    for (int t = tid; t < D * Q * N; t += 128) atomicMax(&mxg[t / (Q * N) * N + t % N], fix_key(vg[t]));
     for (int lf = 0; lf < NF; ++lf) {
         const int code = elem_face[(size_t)e * NF + lf];
         const double* fp = ((code & 1) ? fpsiR : fpsiL) + (size_t)(code >> 1) * QF * N;
         for (int t = tid; t < QF * N; t += 128) a = max(a, fix_key(fp[t]));
     }
-    atomicMax(&mx[0], a);
-    atomicMax(&mx[1], b);
+    atomicMax(&mx, a);
     __syncthreads();
-    const int sa = fix_exp(mx[0]), sb = fix_exp(mx[1]);
-    if (tid == 0) texp[e] = make_int2(sa, sb);
+    const int sa = fix_exp(mx);
+    if (tid == 0) texp[e] = sa;
+    for (int t = tid; t < D * N; t += 128) gexp[(size_t)e * D * N + t] = fix_exp(mxg[t]);
     for (int t = tid; t < Q * N; t += 128) buf[t] = vp[t];
     __syncthreads();
-    for (int t = tid; t < Q * N; t += 128) reinterpret_cast<int2*>(vp)[t] = fix_of(buf[(t % Q) * N + t / Q], sa);
+    for (int t = tid; t < Q * N; t += 128) reinterpret_cast<int2*>(vp)[t] = fix_round(buf[(t % Q) * N + t / Q], sa);
     __syncthreads();
     for (int t = tid; t < D * Q * N; t += 128) buf[t] = vg[t];
     __syncthreads();
     for (int t = tid; t < D * Q * N; t += 128) {
         const int r = GradTab<D, P>::row(t), i = GradTab<D, P>::mode(t);
-        reinterpret_cast<int2*>(vg)[t] = fix_of(buf[((r % D) * Q + r / D) * N + i], sb);
+        reinterpret_cast<int2*>(vg)[t] = fix_round(buf[((r % D) * Q + r / D) * N + i], fix_exp(mxg[r % D * N + i]));
     }
     for (int lf = 0; lf < NF; ++lf) {
         const int code = elem_face[(size_t)e * NF + lf];
@@ -780,7 +843,7 @@ __global__ void __launch_bounds__(128) k_fix_tables(double* __restrict__ vpsi, d
         for (int t = tid; t < QF * N; t += 128) buf[t] = fp[t];
         __syncthreads();
         for (int t = tid; t < QF * N; t += 128)
-            reinterpret_cast<int2*>(fp)[t] = fix_of(buf[FaceTab<D, P>::row(t) * N + FaceTab<D, P>::mode(t)], sa);
+            reinterpret_cast<int2*>(fp)[t] = fix_round(buf[FaceTab<D, P>::row(t) * N + FaceTab<D, P>::mode(t)], sa);
     }
 }
 
@@ -793,7 +856,7 @@ emg_status fix_tables(emg_ctx* c) {
     if constexpr (PP > 0) {                                                                                     \
         EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_fix_tables<DD, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
         ProfScope _ps(c, PC_SETUP);                                                                             \
-        k_fix_tables<DD, PP><<<(unsigned)c->E, 128, sm, c->stream>>>(L.vpsi, L.vgw, c->elem_face, L.fpsiL, L.fpsiR, L.texp); \
+        k_fix_tables<DD, PP><<<(unsigned)c->E, 128, sm, c->stream>>>(L.vpsi, L.vgw, c->elem_face, L.fpsiL, L.fpsiR, L.texp, L.gexp); \
     }
         EMG_DISPATCH_DP(c->dim, p, EMG_FT)
 #undef EMG_FT
@@ -867,7 +930,7 @@ emg_status launch_residual(emg_ctx* c, int p, const double* u, const double* tau
             launch_chained(c, (small ? k_volume<DD, PP, RR, true> : k_volume<DD, PP, RR, false>), (unsigned)((E + ET - 1) / ET), T, 0, \
                 E, u, reinterpret_cast<const int2*>(L.vpsi), reinterpret_cast<const int2*>(L.vgw),             \
                 c->elem_face, reinterpret_cast<const int2*>(L.fpsiL), reinterpret_cast<const int2*>(L.fpsiR),  \
-                L.texp, reinterpret_cast<const int4*>(L.fhat), L.fkey, tau, g, L.vvr, om, R);                                                         \
+                L.texp, L.gexp, reinterpret_cast<const int4*>(L.fhat), L.fkey, tau, g, L.vvr, om, R);                                                         \
         }                                                                                                      \
     }
 #define EMG_RES(DD, PP)                   \

@@ -429,7 +429,7 @@ int64_t estimate_bytes(int dim, int64_t E, int64_t F, int64_t F_int, int p_max, 
         b += 6 * E * B * 8;                                                     // v, v0, tau, un, r, r2
         if (rot) b += (E * Q + F * QF) * 3 * 8;                                 // frame velocities
         if (p > 0) {
-            b += E * 8 + F * (QF * 8 + 5 * 4);                                   // table exponents, fluxes
+            b += E * (1 + dim * N) * 4 + F * (QF * 8 + 5 * 4);                   // table exponents, fluxes
             b += F * QF * 10 * 8 * (blocks_f32(prec) ? 1 : 2);                   // traces
             if (blocks_f32(prec))
                 b += E * B * B * 4 + E * Q * N * (1 + dim) * 4 + F * QF * (N + 25) * 4 + Fi1 * QF * (N + 25) * 4;
@@ -603,7 +603,8 @@ emg_status setup_device_mesh(emg_ctx* c, const emg_mesh_desc* m) {
         EMG_ALLOC(L.fhat, double, F * L.QF * (p > 0 ? 6 : 5));
         if (p > 0) {
             EMG_ALLOC(L.fkey, int, F * 5);
-            EMG_ALLOC(L.texp, int2, E);
+            EMG_ALLOC(L.texp, int, E);
+            EMG_ALLOC(L.gexp, int, E * D * L.N);
             EMG_ALLOC(L.tr, double, F * L.QF * 10);
             L.trj = L.tr;
             if (!blocks_f32(c->prm.prec)) EMG_ALLOC(L.trj, double, F * L.QF * 10);
