@@ -81,6 +81,12 @@ __device__ __forceinline__ int2 fix_shift(int2 p, int k, bool neg) {
     return fix_pair(v);
 }
 
+// (hi, lo) of v 2^-k rounded, k >= 0.
+__device__ __forceinline__ int2 fix_shift_round(int2 p, int k) {
+    const long long v = ((long long)p.x << FIX_LO) + (long long)p.y;
+    return fix_pair(k == 0 ? v : ((v >> min(k - 1, 62)) + 1) >> 1);
+}
+
 // v as a double (v 2^-s is the number it stands for).
 __device__ __forceinline__ double fix_back(int2 v) {
     return __ll2double_rn(((long long)v.x << FIX_LO) + (long long)v.y);

@@ -1,9 +1,17 @@
 // FP64 block assembly (Eq. jac1) on the integer pipe: the element-diagonal blocks of the FP64 form,
 //   D[(a,i),(b,j)] = sum_q psi_j(x_q) s_{ab,i}(q),   s = sum_k W_q d_k psi_i A_k[a][b]  (volume points)
 //                                                    s = -/+ psi_i w|n dS| dF~/dU[a][b]  (face points)
-// as fixed-point sums (fix.cuh): one exponent per element and (a, b) for s, the basis tables' own
-// for psi.  One block per element; thread (ab, i) forms its s of a point from the staged tables and
-// adds s psi_j to the N columns of its row.  Only the pairs (a, b) with an entry other than zero at
+// as fixed-point sums (fix.cuh).  Thread (ab, i) of an element's block forms its s of a point from the
+// staged tables and adds s psi_j to the N columns of its row.  s has 58 bits and an exponent of its
+// own for each (ab, i), from the largest gradients of mode i and Jacobian entries ab; the directions
+// are scaled against each other first (A_k by the power of two of the gradients' size along k), so that
+// the long side of a stretched cell keeps its bits.  psi_j has the bits that the sums leave room for: 2-D
+// 55 (p = 1: 56); 3-D 56, the sums of at most 31 rows going to 96-bit numbers in shared memory.  Error of
+// an entry over its own sum of |terms|, worst and rms in units of 2^-53, CPU emulation (float64 / one
+// exponent a pair (a, b), s cut to 54 bits / this form): 24 x 12 O-grid, p = 4: 5.7, 0.55 / 44, 2.6 / 5.7,
+// 0.39; 128 x 8, p = 3: 4.2, 0.53 / 113, 7.2 / 3.4, 0.30; rectangles of aspect 10^4, p = 4: 5.8, 0.50 /
+// 4400, 136 / 7.3, 0.41; sphere shells, p = 2: 16, 0.84 / 1240, 86 / 11, 0.42, p = 3: 12, 0.90 / 304, 30 /
+// 6.6, 0.56.  Only the pairs (a, b) with an entry other than zero at
 // some point are visited: 17 of 25 in a 2-D flow without a spanwise momentum.  Bound by the integer
 // multiply-adds (3 per term): on the float64 pipe the same sums took 16.7 ms of the FP64 V-cycle of
 // the 128 x 64 O-grid at p = 4.
@@ -20,15 +28,16 @@ struct DiagFx {
     static constexpr int LIVE = D == 2 ? 17 : 25;                      // pairs (a, b) of one pass
     static constexpr int THREADS = (LIVE * N + 31) / 32 * 32;
     static constexpr int NP = (N + 1) & ~1;                            // columns, padded to 16 bytes
-    static constexpr int QC = D == 2 ? Q : 24;                         // volume points per chunk
+    static constexpr int QC = D == 2 || P == 1 ? Q : 24;               // volume points per chunk
     static constexpr int FP = D == 2 ? NF * QF : QF;                   // face points per chunk
     static constexpr int RC = QC > FP ? QC : FP;
-    // sums of at most FIX_TERMS rows keep 56 bits of s; longer ones 54 and fold x into h at the end of
-    // every chunk: |h| <= 512 2^54, |x| <= 200 (2^53 + 2^55)
-    static constexpr bool LONG = Q + NF * QF > FIX_TERMS;
-    // a volume point's s sums D <= 3 products: two bits more
-    static constexpr int SF = LONG ? 2 : 0, SV = SF + 2;
-    static_assert(Q + NF * QF <= 512 && RC <= 100, "exact sums");
+    // bits of s and of the staged psi; over the rows of one sum (3-D: RMAX, then to the 96-bit ones)
+    //   |h| <= rows 2^(SB - 28) 2^(PB - 28) < 2^63,  |x| <= rows (2^(SB - 28) 2^27 + 2^27 2^(PB - 28)) < 2^63
+    static constexpr int SB = 58, PB = D == 2 && P > 1 ? 55 : 56, RMAX = 31;
+    static constexpr int SV = D == 2 ? 1 : 2;                          // bits of a sum of D products
+    static constexpr bool FOLD = D == 2 && N == 15;                    // x into h after the volume points
+    static constexpr int FG = RMAX / QF;                               // 3-D: faces of one sum
+    static_assert((D == 3 && P == 4) || (D == 2 ? Q + FP <= (PB == 56 ? 31 : 62) && (FOLD ? QC : Q + FP) <= 56 : QC <= RMAX && FG >= 1), "exact sums");
     // shared memory (8-byte words); the slab that the rows leave through lies over the tables
     static constexpr int O_PS = 0, O_GS = O_PS + RC * NP, O_AS = O_GS + QC * D * N;
     static constexpr int AW = QC * D > FP ? QC * D : FP;               // rows of 25 entries
@@ -39,7 +48,8 @@ struct DiagFx {
     // resident blocks asked of the register allocator (80 registers a thread in 2-D; 3-D p = 3: 128)
     static constexpr int MINB = D == 2 ? (N == 15 ? 3 : N == 10 ? 4 : 5) : N == 20 ? 1 : N == 10 ? 2 : 4;
     static constexpr int SLAB = N * B;
-    static constexpr size_t SMEM = (size_t)(ALL > SLAB ? ALL : SLAB) * 8;
+    static constexpr int O_ACC = ALL > SLAB ? ALL : SLAB;              // 3-D: [3][N][LIVE N] words of the 96-bit sums
+    static constexpr size_t SMEM = (size_t)O_ACC * 8 + (D == 3 ? (size_t)3 * N * LIVE * N * 4 : 0);
 };
 
 // dF_k/dU (Appendix Eq. dfdu with grad psi -> e_k, omega = 0) less vrk on the diagonal.
@@ -92,17 +102,39 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
     __shared__ double ud[B], Us[Q][5], s_dtau;
     __shared__ int mxa[25], mxj[25], sa[25], sj[25], live[25], nlive;
     const int e = blockIdx.x, tid = threadIdx.x;
-    // the element's exponents of the basis values and, the least of its modes and directions, the gradients
-    __shared__ int ge[D * N];
+    // the gradients' exponents; dk: along k less the least direction's, ty: of mode i after that scaling
+    __shared__ int ge[D * N], dk[D], ty[N], m0;
     for (int t = tid; t < D * N; t += T) ge[t] = gexp[(size_t)e * D * N + t];
     for (int t = tid; t < B; t += T) ud[t] = u[(size_t)e * B + t];
     if (tid < 25) mxa[tid] = mxj[tid] = 0;
-    int2 te = make_int2(texp[e], 0x7fffffff);
+    const int tx = texp[e], tp = tx - (FIX_BITS - C::PB);   // exponents of psi, of the staged psi
     __syncthreads();
-    for (int t = 0; t < D * N; ++t) te.y = min(te.y, ge[t]);
+    if (tid < 32) {
+        int mk[D], least = 0x7fffffff;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            mk[k] = 0x7fffffff;
+            for (int i = tid; i < N; i += 32) mk[k] = min(mk[k], ge[k * N + i]);
+            mk[k] = __reduce_min_sync(0xffffffffu, mk[k]);
+            least = min(least, mk[k]);
+        }
+        for (int i = tid; i < N; i += 32) {
+            int m = 0x7fffffff;
+#pragma unroll
+            for (int k = 0; k < D; ++k) m = min(m, ge[k * N + i] - mk[k]);
+            ty[i] = m;
+#pragma unroll
+            for (int k = 0; k < D; ++k) ge[k * N + i] -= mk[k] + m;   // what is left to shift a staged gradient by
+        }
+        if (tid == 0) {
+            m0 = least;
+#pragma unroll
+            for (int k = 0; k < D; ++k) dk[k] = mk[k] - least;
+        }
+    }
     // U at the volume points (float64: 5 N multiply-adds a point), dtau of Eq. x3d
     {
-        const double sp = fix_scale(-te.x, 0);
+        const double sp = fix_scale(-tx, 0);
         const int2* pv = vpsi + (size_t)e * Q * N;
         for (int t = tid; t < Q * 5; t += T) {
             const int c = t / Q, q = t % Q;
@@ -146,7 +178,8 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
         flux_jac_at(t / D, t % D, A);
 #pragma unroll
         for (int x = 0; x < 25; ++x) {
-            const int k = fix_key(A[x]);
+            int k = fix_key(A[x]);
+            if (k > 0 && k < 0x7ff00000) k = max(k - (dk[t % D] << 20), 1);
             if (k > mxa[x]) atomicMax(&mxa[x], k);
             if (Q == QC) Ad[t * 25 + x] = A[x];
         }
@@ -158,11 +191,8 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
         if (on) live[__popc(m & ((1u << tid) - 1u))] = tid;
         if (tid == 0) nlive = __popc(m);
         if (on) {
-            // one exponent S of s for both kinds of points: s = (table x Jacobian) >> C::SV or C::SF has
-            // exponent te + s_Jacobian - 56 - shift; the kind with the smaller values gives up low bits
-            const int S = min(te.y + fix_exp(mxa[tid]) - C::SV, te.x + fix_exp(mxj[tid]) - C::SF);
-            sa[tid] = S + C::SV - te.y;
-            sj[tid] = S + C::SF - te.x;
+            sa[tid] = fix_exp(mxa[tid]);
+            sj[tid] = fix_exp(mxj[tid]);
         }
     }
     __syncthreads();
@@ -171,21 +201,21 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
         const int2* pv = vpsi + (size_t)e * Q * N + q0;
         for (int t = tid; t < nq * NP; t += T) {
             const int j = t / nq, q = t % nq;
-            ps[q * NP + j] = j < N ? pv[j * Q + q] : make_int2(0, 0);
+            ps[q * NP + j] = j < N ? fix_shift_round(pv[j * Q + q], FIX_BITS - C::PB) : make_int2(0, 0);
         }
         const int2* gv = vgw + (size_t)e * D * Q * N;
         for (int t = tid; t < nq * D * N; t += T) {
             const int r = t / N, i = t % N;
-            gs[t] = fix_shift(gv[GradTab<D, P>::at(q0 * D + r, i)], ge[r % D * N + i] - te.y, false);
+            gs[t] = fix_shift_round(gv[GradTab<D, P>::at(q0 * D + r, i)], ge[r % D * N + i]);
         }
         if (Q == QC) {
-            for (int t = tid; t < Q * D * 25; t += T) As[t] = fix_of(Ad[t], sa[t % 25]);
+            for (int t = tid; t < Q * D * 25; t += T) As[t] = fix_round(Ad[t], sa[t % 25] - dk[t / 25 % D]);
         } else {
             for (int t = tid; t < nq * D; t += T) {
                 double A[25];
                 flux_jac_at(q0 + t / D, t % D, A);
 #pragma unroll
-                for (int x = 0; x < 25; ++x) As[t * 25 + x] = fix_of(A[x], sa[x]);
+                for (int x = 0; x < 25; ++x) As[t * 25 + x] = fix_round(A[x], sa[x] - dk[t % D]);
             }
         }
     };
@@ -194,27 +224,35 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
             const int r = t / NP, j = t % NP;
             const int code = elem_face[(size_t)e * NF + f0 + r / QF];
             const int2* pf = ((code & 1) ? fpsiR : fpsiL) + (size_t)(code >> 1) * QF * N;
-            fs[t] = j < N ? pf[FaceTab<D, P>::at(r % QF, j)] : make_int2(0, 0);
+            fs[t] = j < N ? fix_shift_round(pf[FaceTab<D, P>::at(r % QF, j)], FIX_BITS - C::PB) : make_int2(0, 0);
         }
         for (int t = tid; t < nf * QF * 25; t += T) {
             const int lf = t / (QF * 25), code = elem_face[(size_t)e * NF + f0 + lf];
             const double x = (((code & 1) ? fjr : fjl) + (size_t)(code >> 1) * QF * 25)[t - lf * QF * 25];
-            fj[t] = fix_of((code & 1) ? x : -x, sj[t % 25]);
+            fj[t] = fix_round((code & 1) ? x : -x, sj[t % 25]);
         }
     };
     long long h[N], c[N];
-    int ab = 0, i = 0;
+    int ab = 0, i = 0, kv = 0, kf = 0, ks = 0;   // shifts to s of the products (below), the exponent of s
     bool act = false;
     auto take_row = [&](int pass) {
         const int l = pass * C::LIVE + tid / N;
         act = tid < C::LIVE * N && l < nlive;
         ab = act ? live[l] : 0;
         i = tid % N;
+        // products of the volume (faces) have exponent ev (ef) and, summed over k, 112 + SV (PB + 56) bits;
+        // the kind with the smaller values gives up low bits
+        const int ev = ty[i] + m0 + sa[ab], ef = tp + sj[ab];
+        ks = min(ev - 2 * FIX_BITS - C::SV, ef - FIX_BITS - C::PB) + C::SB;
+        kv = min(ev - ks - 53, 63);
+        kf = min(ef - ks - 53, 63);
 #pragma unroll
         for (int j = 0; j < N; ++j) h[j] = c[j] = 0;
     };
-    auto add_row = [&](long long s, const int2* prow) {
-        const int2 sl = make_int2((int)((s + (1ll << (FIX_LO - 1))) >> FIX_LO), ((int)s << (32 - FIX_LO)) >> (32 - FIX_LO));
+    // s of the exact product h 2^56 + x 2^28, rounded: its upper 60 (+ SV) bits, shifted by k + 1
+    auto add_row = [&](long long ph, long long px, int k, const int2* prow) {
+        const long long t = (((ph << 4) + (px >> (FIX_LO - 4))) >> k) + 1;   // s = t >> 1
+        const int2 sl = make_int2((int)((t + (1ll << FIX_LO)) >> (FIX_LO + 1)), ((int)t << (31 - FIX_LO)) >> (32 - FIX_LO));
         const int4* p4 = reinterpret_cast<const int4*>(prow);
 #pragma unroll
         for (int j = 0; j < N; j += 2) {
@@ -229,7 +267,7 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
             long long sh = 0, sx = 0;
 #pragma unroll
             for (int k = 0; k < D; ++k) fix_mac(sh, sx, gs[(q * D + k) * N + i], As[(q * D + k) * 25 + ab]);
-            add_row((sh + (sx >> FIX_LO)) >> C::SV, ps + q * NP);
+            add_row(sh, sx, kv, ps + q * NP);
         }
     };
     auto mac_faces = [&](int np) {
@@ -237,14 +275,32 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
         for (int t = 0; t < np; ++t) {
             long long sh = 0, sx = 0;
             fix_mac(sh, sx, fs[t * NP + i], fj[t * 25 + ab]);
-            add_row((sh + (sx >> FIX_LO)) >> C::SF, fs + t * NP);
+            add_row(sh, sx, kf, fs + t * NP);
         }
     };
     auto fold = [&]() {
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            h[j] += c[j] >> FIX_LO;
+            h[j] += (c[j] + (1ll << (FIX_LO - 1))) >> FIX_LO;
             c[j] = 0;
+        }
+    };
+    // 3-D: the sums so far to this thread's 96-bit ones (words [3][N][LIVE N], one thread's apart from another's)
+    unsigned* acc = reinterpret_cast<unsigned*>(sm + C::O_ACC) + tid;
+    constexpr int AN = C::LIVE * N;
+    auto flush = [&](bool first) {
+        fold();
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            unsigned lo = (unsigned)h[j], mid = (unsigned)(h[j] >> 32), hi = (unsigned)(h[j] >> 63);
+            if (!first)
+                asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+                    : "+r"(lo), "+r"(mid), "+r"(hi)
+                    : "r"(acc[j * AN]), "r"(acc[(N + j) * AN]), "r"(acc[(2 * N + j) * AN]));
+            acc[j * AN] = lo;
+            acc[(N + j) * AN] = mid;
+            acc[(2 * N + j) * AN] = hi;
+            h[j] = 0;
         }
     };
     double* slab = reinterpret_cast<double*>(smraw);
@@ -259,6 +315,7 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
     if constexpr (D == 2) {
         if (act) {
             mac_volume(Q);
+            if (C::FOLD) fold();
             mac_faces(FP);
         }
     } else {
@@ -268,24 +325,34 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
             if (q0 > 0) __syncthreads();
             stage_volume(q0, nq);
             __syncthreads();
-            if (act) mac_volume(nq);
-            if (act && C::LONG) fold();
+            if (act) {
+                mac_volume(nq);
+                flush(q0 == 0);
+            }
         }
 #pragma unroll 1
         for (int lf = 0; lf < NF; ++lf) {
             __syncthreads();
             stage_faces(lf, 1);
             __syncthreads();
-            if (act) mac_faces(QF);
-            if (act && C::LONG) fold();
+            if (act) {
+                mac_faces(QF);
+                if ((lf + 1) % C::FG == 0 || lf + 1 == NF) flush(false);
+            }
         }
     }
     // this thread's N entries of its row to `row`: D, or P = I/dtau - D
     auto put_row = [&](double* row) {
-        const double scale = fix_scale(2 * FIX_BITS - te.x - (te.x + sj[ab] - C::SF), max(mxa[ab], mxj[ab]));
+        const double scale = fix_scale(FIX_BITS - ks - tp, max(mxa[ab], mxj[ab]));
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            const double v = fix_sum(h[j], c[j], scale);
+            double v;
+            if constexpr (D == 2) {
+                v = fix_sum(h[j], c[j], scale);
+            } else {
+                const long long up = (long long)(((unsigned long long)acc[(2 * N + j) * AN] << 32) | acc[(N + j) * AN]);
+                v = fma(__ll2double_rn(up), 4294967296.0, (double)acc[j * AN]) * scale;
+            }
             row[j] = shifted ? ((ab % 6 == 0 && i == j) ? idt : 0.0) - v : v;   // ab % 6 == 0: a == b
         }
     };
@@ -300,6 +367,7 @@ __global__ void __launch_bounds__(DiagFx<D, P>::THREADS, DiagFx<D, P>::MINB) k_d
         take_row(1);
         if (act) {
             mac_volume(Q);
+            if (C::FOLD) fold();
             mac_faces(FP);
             put_row(blk + (size_t)(ab / 5 * N + i) * B + ab % 5 * N);
         }
