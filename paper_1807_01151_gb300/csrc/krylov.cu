@@ -15,6 +15,7 @@
 #include <functional>
 #include <mutex>
 
+#include "arnoldi_blocks.h"
 #include "common.cuh"
 
 namespace cg = cooperative_groups;
@@ -61,23 +62,6 @@ __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned nblocks, unsign
 
 constexpr int ARN_THREADS = 256;
 
-// Blocks of the Arnoldi process, at most `cap` and what is co-resident (per_sm per SM; two, as the form with
-// rows in registers).  More blocks share out the rows' work, fewer make the cross-block reductions
-// shorter, which every block repeats.  Measured, us of an EXP1 step (m = 30) with 64, 128, 192 and 256 rows a
-// block: float64, whose pipe a block of 256 rows fills, 2560 rows 739 747 801 872, 10240 rows 887 756 806
-// 880, 23040 rows 1111 1132 840 905, 40960 rows 1319 (304 blocks) 1322 1352 1384; float32 2560 rows 478
-// 479 495 491, 10240 rows 511 487 496 490, 23040 rows 669 585 525 518, 40960 rows 717 720 664 619.
-template <class T>
-static int64_t arnoldi_blocks(int64_t K0, int nsm, int per_sm, int64_t cap) {
-    auto blocks = [K0](int64_t rows) { return (K0 + rows - 1) / rows; };
-    const int64_t resident = (int64_t)nsm * std::max(1, std::min(per_sm, 2));
-    int64_t nb;
-    if (sizeof(T) == 4)
-        nb = blocks(K0 <= 10240 ? 128 : 256);
-    else
-        nb = blocks(128) <= nsm ? blocks(128) : blocks(192) <= nsm ? blocks(192) : resident;
-    return std::max<int64_t>(1, std::min({nb, resident, cap}));
-}
 constexpr int ARN_CHUNK = 8;  // vectors per dot-product sweep
 static_assert(ARN_CHUNK == 8, "warp_sum8 reduces eight columns");
 
@@ -1057,7 +1041,7 @@ static emg_status exp1_krylov(emg_ctx* c, const double* u0, const double* dt, do
     EMG_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_arnoldi<T>, ARN_THREADS, 0));
     EMG_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_rv, k_arnoldi_rv<T, ARN_RV>, ARN_THREADS, 0));
     EMG_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    const int64_t nb = arnoldi_blocks<T>(K0, nsm, per_sm, c->red_blocks);
+    const int64_t nb = arnoldi_blocks(K0, sizeof(T) == 4, nsm, per_sm, c->red_blocks);
     // rows in registers: one row per thread at most, every block co-resident, m <= ARN_RV
     const bool rows_in_regs = m <= ARN_RV && (K0 + nb - 1) / nb <= ARN_THREADS && nb <= (int64_t)nsm * per_sm_rv;
     const int stride = MAX_KRYLOV + 8;
@@ -1244,7 +1228,7 @@ extern "C" emg_status emg_exp1_step_noalloc(int32_t dim, int64_t n_elems, const 
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_arnoldi<double>, ARN_THREADS, 0) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return EMG_ERR_CUDA;
-    const int64_t nb = arnoldi_blocks<double>(K0, nsm, per_sm, NA_BLOCKS);
+    const int64_t nb = arnoldi_blocks(K0, false, nsm, per_sm, NA_BLOCKS);
     int64_t K0a = K0;
     int Ea = (int)E, NFa = NF, ma = krylov_m, stra = NA_STRIDE;
     const double* bsrc = bsr;
