@@ -42,11 +42,11 @@ struct GjWork {
 };
 inline GjWork gj_work(int* w, int64_t E) { return {w, w + E, w + 4 * E, w + 2 * E, w + 3 * E, w + 4 * E + 2}; }
 
-// Length of a list, read by every CTA of a grid; the last one out sets it back to 0.
+// Length of a list, read by every CTA of a grid; the last one out sets it back to 0 (an empty one is 0).
 __device__ __forceinline__ int take_list(int* head) {
     const int n = *reinterpret_cast<volatile int*>(head);
     __syncthreads();   // every thread has read it
-    if (threadIdx.x == 0) {
+    if (n > 0 && threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(head + 1, 1) == (int)gridDim.x - 1) {   // every CTA has
             head[0] = 0;
@@ -55,7 +55,14 @@ __device__ __forceinline__ int take_list(int* head) {
     }
     return n;
 }
-constexpr unsigned kListBlocks = 608;   // CTAs that share a list: four per SM
+// CTAs that share a list: enough for 32 warps an SM (four CTAs at least, 16 at most), so that a level whose
+// blocks are all listed (a 2-D flow with a spanwise momentum) fills the chip.  Smoothing step of 128 x 64,
+// float32 blocks, all listed, with 4 CTAs an SM / as here: p = 1 470 / 375 us, p = 2 629 / 530 us; none
+// listed 321 / 322 us and 379 / 382 us.
+inline unsigned list_grid(int64_t E, int threads) {
+    const int64_t per_sm = threads >= 256 ? 4 : threads <= 64 ? 16 : 1024 / threads, n = 152 * per_sm;
+    return (unsigned)(E < n ? E : n);
+}
 
 // B = 5 N(p): 2-D p = 1..4, then 3-D p = 1..4 (B = 50 serves both dimensions).
 #define EMG_BSIZES(X) X(15) X(30) X(50) X(75) X(20) X(100) X(175)

@@ -357,7 +357,9 @@ __global__ void __launch_bounds__(32 * W, GjSplit<N, W>::MINB) k_gj_split(
     if (threadIdx.x < 32) invk3[threadIdx.x] = -1;
     float* out = blk + gj_packed_at(e, B);
     bool coupled = false;
-    if (asm_flag && asm_flag[e]) {
+    if (asm_flag && !asm_flag[e]) {   // left whole by the assembly, which found it coupled
+        coupled = true;
+    } else if (asm_flag) {
 #pragma unroll 8
         for (int t = threadIdx.x; t < B4 * B4; t += T) tile[t / B4 * LD + t % B4] = out[t];
         for (int t = threadIdx.x; t < N * N; t += T) s3[t] = out[B4 * B4 + t];
@@ -499,7 +501,7 @@ static cudaError_t gj_split_launch(int v, unsigned E, float* blk, const GjWork& 
     static_assert(G::VALID, "the blocked form serves every 2-D block");
     e = cudaFuncSetAttribute(k_gj_blk<5 * N, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
     if (e != cudaSuccess) return e;
-    k_gj_blk<5 * N, 4><<<E < kListBlocks ? E : kListBlocks, 128, G::SMEM, st>>>((int)E, blk, k.list, k.head);
+    k_gj_blk<5 * N, 4><<<list_grid(E, 128), 128, G::SMEM, st>>>((int)E, blk, k.list, k.head);
     return cudaGetLastError();
 }
 // packed: the blocks come from the plane assembly.

@@ -137,6 +137,13 @@ __global__ void __launch_bounds__(160, DiagPl<P>::MINB) k_diag_blocks_pl(
             bad[el] = 1;
     }
     __syncthreads();
+    if (__all_sync(0xffffffffu, (tid & 31) >= ne || bad[tid & 31])) {   // nothing to sum: all on the list
+        if (tid < ne) {
+            flag[e0 + tid] = 0;
+            list[atomicAdd(head, 1)] = e0 + tid;
+        }
+        return;
+    }
     const int sw = tid - 128;   // >= 0: spanwise row
     const int el = sw < 0 ? tid / B4 : sw / N;
     const int a4 = sw < 0 ? tid % B4 / N : 0, i = sw < 0 ? tid % N : sw % N;

@@ -601,7 +601,6 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
             st = launch_diag_blocks_plane(c, p, u, cfl_dev, shifted, out);
             if (st != EMG_OK) return st;
         }
-        const unsigned grid = L.asm_plane ? (unsigned)std::min<int64_t>(c->E, kListBlocks) : (unsigned)c->E;
 #define EMG_DB32(DD, PP)                                                                                    \
     if constexpr (PP > 0) {                                                                                 \
         EMG_CUDA_TRY(c, cudaFuncSetAttribute(k_diag_blocks_rb<DD, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
@@ -612,7 +611,8 @@ emg_status launch_diag_blocks32(emg_ctx* c, int p, const double* u, const double
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
                 c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, nullptr, nullptr, out);               \
         else                                                                                                \
-            k_diag_blocks_rb<DD, PP><<<grid, DiagRb<DD, PP>::THREADS, DiagRb<DD, PP>::SM * 4, c->stream>>>( \
+            k_diag_blocks_rb<DD, PP><<<L.asm_plane ? list_grid(c->E, DiagRb<DD, PP>::THREADS) : (unsigned)c->E, \
+                                       DiagRb<DD, PP>::THREADS, DiagRb<DD, PP>::SM * 4, c->stream>>>(       \
                 (int)c->E, nmax, u, L.vpsi32, L.vgw32, c->elem_face, L.fpsiL32, L.fpsiR32, L.fjl32, L.fjr32,  \
                 c->psic, c->h, cfl_dev, c->prm.gamma, shifted, L.vvr, out,                                  \
                 L.asm_plane ? w.asm_list : nullptr, w.asm_head);                                            \

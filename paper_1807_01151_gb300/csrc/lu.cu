@@ -563,7 +563,7 @@ static emg_status lu_split(emg_ctx* c, LevelDev& L) {
     }
     EMG_CHECK_LAUNCH(c);
     ProfScope _ps(c, PC_LU);
-    k_lu<5 * N><<<E < kListBlocks ? E : kListBlocks, LuCfg<5 * N>::THREADS, LuCfg<5 * N>::SMEM, c->stream>>>(
+    k_lu<5 * N><<<list_grid(c->E, LuCfg<5 * N>::THREADS), LuCfg<5 * N>::THREADS, LuCfg<5 * N>::SMEM, c->stream>>>(
         (int)E, L.blk, L.piv, L.lu_list, L.lu_list + E);
     EMG_CHECK_LAUNCH(c);
     return EMG_OK;
