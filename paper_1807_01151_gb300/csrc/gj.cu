@@ -578,14 +578,26 @@ __global__ void k_fill_tuning_blocks(int64_t n, int B, bool split, float* __rest
     const bool zero = split && (r / (B / 5) == 3) != (c / (B / 5) == 3);
     blk[t] = zero ? 0.0f : (r == c ? (float)B : 0.0f) + ((float)(h & 0xffffu) / 65536.0f - 0.5f);
 }
+// The same, packed as the plane assembly leaves them (blocks.cuh).
+__global__ void k_fill_tuning_packed(int64_t n, int N, float* __restrict__ blk) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int B4 = 4 * N, len = 17 * N * N;
+    if (t >= n * len) return;
+    const int o = (int)(t % len), m = o < B4 * B4 ? B4 : N, q = o < B4 * B4 ? o : o - B4 * B4;
+    const uint32_t h = (uint32_t)(t * 2654435761ull) ^ (uint32_t)(t >> 13);
+    blk[gj_packed_at(t / len, 5 * N) + o] = (q / m == q % m ? 5.0f * N : 0.0f) + ((float)(h & 0xffffu) / 65536.0f - 0.5f);
+}
 
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int>, int> g_gj_best;   // (device, B, family) -> variant
+std::map<std::tuple<int, int, int, int>, int> g_gj_best;   // (device, B, family, log2 of the stand-ins) -> variant
 }  // namespace
 
-// Times every valid variant on min(E, 2048) stand-in blocks per block size of the FP32 levels
-// and keeps the fastest, once per (device, B) for the process.
+// Times every valid variant per block size of the FP32 levels on as many stand-in blocks as the level
+// has, at most 2048 (32 MB of small ones), packed where the level's own come packed from the assembly, and
+// keeps the fastest, once per (device, B, family, power of two of their number) for the process.  Whole
+// stand-ins in the place of packed ones chose other variants (128 x 64, p = 4: a smoothing step 1030 us, now
+// 946), and so did 512 blocks of B = 15 for 8192 (p = 1: 322 us with 8 warps, 303 with 4).
 emg_status tune_gj(emg_ctx* c) {
     if (!blocks_f32(c->prm.prec)) return EMG_OK;
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -594,7 +606,11 @@ emg_status tune_gj(emg_ctx* c) {
         // the split form serves 2-D levels unless the tensor-core or unblocked forms are asked for
         L.gj_split = c->dim == 2 && !L.tc_gj && c->prm.block_kernels != 3;
         L.asm_plane = L.gj_split && !L.tc_asm && !c->rot;
-        const auto key = std::make_tuple(c->device, L.B, L.gj_split ? 2 : (int)(c->prm.block_kernels == 3));
+        const bool packed = L.asm_plane;
+        const int64_t n = std::min<int64_t>(c->E, std::max(2048, (8 << 20) / (L.B * L.B)));
+        int class_n = 0;
+        while (n >> (class_n + 1)) ++class_n;
+        const auto key = std::make_tuple(c->device, L.B, packed ? 3 : L.gj_split ? 2 : (int)(c->prm.block_kernels == 3), class_n);
         if (L.gj_split)   // the list's length and ticket (piv holds the FP64 form's pivots only)
             EMG_CUDA_TRY(c, cudaMemsetAsync(L.piv, 0, (size_t)c->E * L.B * sizeof(int), c->stream));
         // the family: blocked where a blocked variant is valid (unless the unblocked forms are
@@ -606,7 +622,8 @@ emg_status tune_gj(emg_ctx* c) {
         const int v_hi = L.gj_split ? 4 : blocked ? kGjVariants : kGjBlkFirst;   // 0..3 / 14..17 / 0..13
         auto valid = [&](int v) { return L.gj_split ? gj_split_ok(L.B, v) : gj_valid(L.B, v); };
         auto name = [&](int v) {
-            return L.gj_split ? "split " + std::to_string(kGjBlkWarps[v]) + " warps" : gj_variant_name(v);
+            return L.gj_split ? (packed ? "packed split " : "split ") + std::to_string(kGjBlkWarps[v]) + " warps"
+                              : gj_variant_name(v);
         };
         if (!c->prm.autotune) {
             L.gj_variant = 0;
@@ -628,11 +645,16 @@ emg_status tune_gj(emg_ctx* c) {
                          " (tuned earlier in this process); ";
             continue;
         }
-        const int64_t n = std::min<int64_t>(c->E, 2048);
         float* scratch = nullptr;
         EMG_CUDA_TRY(c, cudaMallocAsync((void**)&scratch, (size_t)n * L.B * L.B * sizeof(float), c->stream));
-        const unsigned fill = (unsigned)((n * L.B * L.B + 255) / 256);
-        k_fill_tuning_blocks<<<fill, 256, 0, c->stream>>>(n, L.B, L.gj_split, scratch);
+        auto fill = [&]() {
+            if (packed)
+                k_fill_tuning_packed<<<(unsigned)((n * 17 * L.N * L.N + 255) / 256), 256, 0, c->stream>>>(n, L.N, scratch);
+            else
+                k_fill_tuning_blocks<<<(unsigned)((n * L.B * L.B + 255) / 256), 256, 0, c->stream>>>(n, L.B, L.gj_split, scratch);
+        };
+        fill();
+        if (packed) EMG_CUDA_TRY(c, cudaMemsetAsync(gj_work(L.piv, n).asm_flag, 1, n * sizeof(int), c->stream));
         cudaEvent_t e0, e1;
         EMG_CUDA_TRY(c, cudaEventCreate(&e0));
         EMG_CUDA_TRY(c, cudaEventCreate(&e1));
@@ -645,10 +667,10 @@ emg_status tune_gj(emg_ctx* c) {
             float ms = 1e30f;
             for (int rep = 0; rep < 3 && ok; ++rep) {
                 if (L.gj_split)   // the inverses left packed are no split blocks
-                    k_fill_tuning_blocks<<<fill, 256, 0, c->stream>>>(n, L.B, true, scratch);
+                    fill();
                 EMG_CUDA_TRY(c, cudaEventRecord(e0, c->stream));
                 if (L.gj_split)
-                    EMG_CUDA_TRY(c, gj_split_dispatch(L.B, v, (unsigned)n, scratch, L.piv, false, c->stream));
+                    EMG_CUDA_TRY(c, gj_split_dispatch(L.B, v, (unsigned)n, scratch, L.piv, packed, c->stream));
                 else
                     EMG_CUDA_TRY(c, gj_dispatch(L.B, v, (unsigned)n, scratch, c->stream, &ok));
                 EMG_CUDA_TRY(c, cudaEventRecord(e1, c->stream));
