@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(TrCfg<D, P>::THREADS) k_traces(int E, const do
 // The Roe flux of euler.cuh's roe_flux in float64, scaled by am, with four special functions
 // instead of seven: one reciprocal for both densities, sqrt(rho_R / rho_L) for the averages (weights
 // 1 / (1 + s) and s / (1 + s)), and one reciprocal square root for c and 1 / c^2.  The jumps are
-// differences of rounded numbers (not fused with the product before them), so that equal states have
+// differences of rounded numbers (not fused with the product before them; the pressure's from the
+// internal energies, where it rounds least), so that equal states have
 // none: the flux along a wall or through a uniform flow is free of dissipation to the last bit.  NK = 2:
 // a face in the x-y plane between states without a z momentum (every z term is 0).
 template <int NK, bool ROT>
@@ -155,7 +156,8 @@ __device__ __forceinline__ void roe_flux_fast(const double UL[5], const double U
         qR = fma(vR, n[k], qR);
         dv[k] = __dsub_rn(vR, vL[k]);
     }
-    const double pL = (g - 1.0) * fma(-0.5, kL, UL[4]), pR = (g - 1.0) * fma(-0.5, kR, UR[4]);
+    const double iL = fma(-0.5, kL, UL[4]), iR = fma(-0.5, kR, UR[4]);   // p / (g - 1)
+    const double pL = (g - 1.0) * iL, pR = (g - 1.0) * iR;
     const double EL = UL[4] + pL, ER = UR[4] + pR;
     const double HL = EL * irL, HR = ER * irR;
     const double s2 = ratio_or_negative(UR[0], irL, UL[0]);
@@ -174,7 +176,7 @@ __device__ __forceinline__ void roe_flux_fast(const double UL[5], const double U
     const double c = c2 * ic, ic2 = ic * ic;
     const double dqn = qR - qL;
     const double qn = fma(wR, dqn, qL);
-    const double drho = UR[0] - UL[0], dp = __dsub_rn(pR, pL);
+    const double drho = UR[0] - UL[0], dp = (g - 1.0) * (iR - iL);
     const double rq = rho * c * dqn, hc = 0.5 * ic2;
     const double qr = ROT ? qn - vrn : qn;
     const double l2 = fabs(qr);
