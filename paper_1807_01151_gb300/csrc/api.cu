@@ -9,6 +9,7 @@
 
 #include "blocks.cuh"
 #include "common.cuh"
+#include "residual_chain.h"
 
 using namespace emg;
 
@@ -640,11 +641,9 @@ emg_status emg_residual(emg_ctx* c, int32_t p, const double* u, double* R, int32
         st = stage_out(c, n, &Rd);
         if (st != EMG_OK) return st;
     }
-    // short kernels of one residual follow each other closely (common.cuh); the line is by the basis
-    // table's entries: 4.4 million of 128 x 64 at p = 4 gain 3 %, 24 million of 3234 hexes lose 1 %
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     EMG_CUDA_TRY(c, cudaStreamIsCapturing(c->stream, &cap));
-    c->chain = c->E * c->lv[p].N * c->lv[p].Q <= 8000000 && !c->prof.on && cap == cudaStreamCaptureStatusNone;
+    c->chain = residual_chains(c->dim, p, c->E, c->F * c->lv[p].QF) && !c->prof.on && cap == cudaStreamCaptureStatusNone;
     emg_status st = launch_residual(c, p, ud, nullptr, Rd);
     c->chain = false;
     if (st != EMG_OK) return st;

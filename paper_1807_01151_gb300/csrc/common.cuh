@@ -241,8 +241,7 @@ namespace emg {
 // while the last blocks of the kernel before it still run, and chain_wait, which every such kernel calls
 // before it touches memory, returns when that kernel has completed (all of its chain then has, since
 // each of them waited too).  Saves the launch latency and ramp between the kernels of a residual called by
-// itself: 32 x 16 p = 1 10.9 -> 8.3 us, 128 x 64 p = 4 83.3 -> 80.5 us.  Not used for larger ones (3234
-// hexes at p = 4: 502 against 509 us) nor inside a smoothing step or cycle, where blocks that wait hold
+// itself, where residual_chain.h says so; not used inside a smoothing step or cycle, where blocks that wait hold
 // places that other kernels could use (128 x 64 mixed V-cycle 6.22 against 6.44 ms): emg_ctx::chain.
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

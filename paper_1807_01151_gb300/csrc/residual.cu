@@ -27,6 +27,7 @@
 #include "dispatch.cuh"
 #include "euler.cuh"
 #include "fix.cuh"
+#include "residual_chain.h"
 
 namespace emg {
 
@@ -368,6 +369,7 @@ struct VolCfg {
     static constexpr int TM = L::N * PARTS;                          // threads of an element's projection
     static constexpr int THREADS = S ? (TM <= 64 ? 64 : (TM + 31) / 32 * 32) : (D == 2 || L::N == 20) ? 64 : 128;
     static constexpr int ET = THREADS / TM;                          // elements per block
+    static_assert(S || P == 0 || ET == volume_elems(D, P), "residual_chain.h");
     static constexpr int FS = 6;                                     // padded variable stride
     static constexpr int QMAX = 54;                                  // points of one exact sum (more: no faster)
     static constexpr int QS = THREADS * 288 / (ET * D * FS * 8);     // points that fit the buffer
