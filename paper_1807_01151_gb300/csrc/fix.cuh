@@ -53,6 +53,14 @@ __device__ __forceinline__ int2 fix_pair(long long v) {
     return make_int2((int)((v + (1ll << (FIX_LO - 1))) >> FIX_LO), ((int)v << (32 - FIX_LO)) >> (32 - FIX_LO));
 }
 
+// The same with FIX_NAN in the place of an exponent for a group that holds an infinity or a NaN (e is
+// then above any number's).
+constexpr int FIX_NAN = -100000;
+__device__ __forceinline__ double fix_scale(int e) {
+    const int b = 1023 + e;
+    return b >= 2047 ? __hiloint2double(b > 50000 ? 0x7ff80000 : 0x7ff00000, 0) : b <= 0 ? 0.0 : __hiloint2double(b << 20, 0);
+}
+
 // v = x 2^s cut to an integer, as (hi, lo); |x| 2^s < 2^56.
 __device__ __forceinline__ int2 fix_of(double x, int s) {
     const int hw = __double2hiint(x);

@@ -373,8 +373,8 @@ struct VolCfg {
     static constexpr int FS = 6;                                     // padded variable stride
     static constexpr int QMAX = 54;                                  // points of one exact sum (more: no faster)
     static constexpr int QS = THREADS * 288 / (ET * D * FS * 8);     // points that fit the buffer
-    static constexpr int QC0 = (QS < QMAX ? QS : QMAX) & ~1;
-    static constexpr int QC = QC0 < L::Q ? QC0 : L::Q;               // points per chunk
+    static constexpr int QC0 = QS < QMAX ? QS : QMAX;
+    static constexpr int QC = QC0 < L::Q ? QC0 & ~1 : L::Q;          // points per chunk (even, or all)
     static constexpr int FC0 = (QC * D) / L::QF;                     // faces that fit the same buffer
     static constexpr int FC1 = FC0 < FIX_TERMS / L::QF ? FC0 : FIX_TERMS / L::QF;
     static constexpr int FC = FC1 < 1 ? 1 : (FC1 > L::NF ? L::NF : FC1);
@@ -382,7 +382,6 @@ struct VolCfg {
     static constexpr int SH = D * QC > 252 ? 2 : D * QC > 120 ? 1 : 0;
     static constexpr int ROWS = QC * D > FC * L::QF ? QC * D : FC * L::QF;
     static constexpr int MINB = 512 / THREADS;                       // 128 registers a thread
-    static constexpr int KB = QC < L::Q ? 2 : 1;                     // buffers of the stages' keys
     static_assert(QC >= 2 && FC * L::QF <= FIX_TERMS && QC <= FIX_TERMS && D * QC <= 504 && L::N <= FIX_TERMS, "exact sums");
 };
 
@@ -539,13 +538,12 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
     constexpr int RV = Q == QC ? Q * D : 0;   // rows of the volume term when it is one chunk
     __shared__ __align__(16) int2 us[ET * N * FS];          // [ET][N][6] coefficients
     __shared__ __align__(16) double Fs[ET * ROWS * FS];     // [ET][rows][6] staged fluxes
-    __shared__ int mxu[ET * 5], mx[CF::KB][ET * D * 5];   // largest keys, of a stage and the next
-    __shared__ int codes[ET * NF];
+    __shared__ int mxu[ET * 5], mx[ET * D * 5];           // largest keys, of a chunk
+    __shared__ int codes[ET * NF], ex[ET * D * 5];          // ex: exponents of the stage's fluxes
     const int e0 = blockIdx.x * ET;
     for (int t = threadIdx.x; t < ET * D * 5; t += T) {
         if (t < ET * 5) mxu[t] = 0;
-#pragma unroll
-        for (int s = 0; s < CF::KB; ++s) mx[s][t] = 0;
+        mx[t] = 0;
     }
     for (int t = threadIdx.x; t < ET * NF; t += T)
         codes[t] = e0 + t / NF < E ? elem_face[(size_t)e0 * NF + t] : 0;
@@ -574,7 +572,6 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
     const int e2 = e0 + el2;
     const bool own = el2 < ET && e2 < E;
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    int stage = 0;   // which of the keys' buffers
     // exact sums to acc: the scale is 2^(56 - s_table - s_flux), NaN for a non-finite flux
     auto add_sums = [&](const long long* h, const long long* c, int st, const int* keys, bool w) {
 #pragma unroll
@@ -585,11 +582,9 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
         }
     };
 #pragma unroll 1
-    for (int q0 = 0; q0 < Q; q0 += QC, stage ^= CF::KB - 1) {
+    for (int q0 = 0; q0 < Q; q0 += QC) {
         const int nq = (Q - q0) < QC ? (Q - q0) : QC;
         __syncthreads();   // us staged / previous chunk consumed
-        if (q0 > 0)
-            for (int t = threadIdx.x; t < ET * D * 5; t += T) mx[stage ^ 1][t] = 0;   // for the next one
         // (1) U_h and the Euler flux at the chunk's points
         for (int t = threadIdx.x; t < ET * nq; t += T) {
             const int el = t / nq, qq = t % nq, e = e0 + el;
@@ -642,12 +637,14 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
                 for (int a = 0; a < 5; ++a) key[k * 5 + a] = fix_key(Fk[a]);
                 row_put(Fs + ((size_t)el * nq * D + qq * D + k) * FS, Fk);
             }
-            row_max<D * 5>(mx[stage], el, key);
+            row_max<D * 5>(mx, el, key);
         }
         __syncthreads();
+        for (int t = threadIdx.x; t < ET * D * 5; t += T) ex[t] = mx[t] >= 0x7ff00000 ? FIX_NAN : fix_exp(mx[t]);
         for (int t = threadIdx.x; t < ne * D * nq; t += T)
-            row_fix<D>(Fs + (size_t)t * FS, mx[stage] + (t / (D * nq) * D + t % D) * 5);
+            row_fix<D>(Fs + (size_t)t * FS, mx + (t / (D * nq) * D + t % D) * 5);
         __syncthreads();
+        for (int t = threadIdx.x; t < ET * D * 5; t += T) mx[t] = 0;   // for the next chunk
         // (2) projection on the gradients: sum_q sum_k W_q d_k psi_i F_k,a
         if (own) {
             long long h[D * 5], c[D * 5];
@@ -655,11 +652,11 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
             for (int a = 0; a < D * 5; ++a) h[a] = c[a] = 0;
             const int2* tab = vgw + (size_t)e2 * D * Q * N + (size_t)q0 * D * N + 2 * i2;
             const double* row = Fs + (size_t)el2 * nq * D * FS;
-            const int* keys = mx[stage] + el2 * D * 5;
+            const int* e5 = ex + el2 * D * 5;
             int rows = nq * D, ge[D];
 #pragma unroll
             for (int k = 0; k < D; ++k) ge[k] = gexp[((size_t)e2 * D + k) * N + i2];
-            const bool w = D == 3 || (keys[3] | keys[8]) != 0;
+            const bool w = D == 3 || e5[3] != fix_exp(0) || e5[8] != fix_exp(0);
             if (w)
                 rows_mac<true, D, N, GT::paired, PARTS, RV>(h, c, tab, row, rows, part);
             else
@@ -674,18 +671,16 @@ __global__ void __launch_bounds__(VolCfg<D, P, S>::THREADS, VolCfg<D, P, S>::MIN
 #pragma unroll
             for (int a = 0; a < 5; ++a) {
                 if (a == 3 && !w) continue;
-                int ek[D], lo = 0x7fffffff, key = 0;
+                int ek[D], lo = 0x7fffffff;
 #pragma unroll
                 for (int k = 0; k < D; ++k) {
-                    ek[k] = ge[k] + fix_exp(keys[k * 5 + a]);
+                    ek[k] = ge[k] + e5[k * 5 + a];
                     lo = min(lo, ek[k]);
-                    key = max(key, keys[k * 5 + a]);
                 }
                 long long s = 0;
 #pragma unroll
-                for (int k = 0; k < D; ++k)
-                    s += (h[k * 5 + a] + ((c[k * 5 + a] + (1ll << (FIX_LO - 1))) >> FIX_LO)) >> min(ek[k] - lo + CF::SH, 63);
-                acc[a] += __ll2double_rn(s) * fix_scale(FIX_BITS + CF::SH - lo, key);
+                for (int k = 0; k < D; ++k) s += (h[k * 5 + a] + (c[k * 5 + a] >> FIX_LO)) >> min(ek[k] - lo + CF::SH, 63);
+                acc[a] += __ll2double_rn(s) * fix_scale(FIX_BITS + CF::SH - lo);
             }
         }
     }
