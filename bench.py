@@ -273,6 +273,24 @@ def kernel_rooflines(prof_cycle, work, peaks, hbm_gbs, form):
     return out
 
 
+def unit_roofline(ops, seconds, peaks, hbm_gbs):
+    """The unit that needs longest for these operations, its rate and the fraction of its peak."""
+    from paper_1807_01151_gb300 import perfmodel
+    t = perfmodel.unit_times(ops, peaks, hbm_gbs)
+    unit = max(t, key=t.get)
+    frac = t[unit] / seconds
+    peak, name = {"int": (perfmodel.INT_MAD_TOPS, "T integer multiply-adds/s"), "f64": (peaks["fp64_tflops"], "TFLOP/s"),
+                  "f32": (peaks["fp32_tflops"], "TFLOP/s"), "hbm": (hbm_gbs, "GB/s")}[unit]
+    return {"bound": "hbm" if unit == "hbm" else "alu", "pipe": unit, "achieved": frac * peak, "peak": peak, "unit": name,
+            "frac": frac}
+
+
+def unit_rooflines(prof_cycle, work, peaks, hbm_gbs):
+    """unit_roofline of every kernel class of a cycle (perfmodel.kernel_work)."""
+    return {k: dict(unit_roofline(work[k], v["ms_per_cycle"] * 1e-3, peaks, hbm_gbs), ms_per_cycle=v["ms_per_cycle"])
+            for k, v in prof_cycle.items() if k in work and v["ms_per_cycle"] > 0}
+
+
 def measure(pkg, torch, mesh, W, prec, args, world, local, rank, with_clocks, peaks, hbm_gbs):
     """Time K V-cycles of one form; return a dict of results (and the solver closed)."""
     import numpy as np
@@ -395,19 +413,20 @@ def measure(pkg, torch, mesh, W, prec, args, world, local, rank, with_clocks, pe
             out["start_spread"] = {"starts": "free stream, then the free stream times (1 + 1e-13 z), z seeded normal",
                                    "cycles": cyc, "seconds": [None if x is None else round(x, 3) for x in sec],
                                    "median_s": float(np.median(ok)) if ok else None}
-    # roofline of the dominant FP64 kernel, k_volume at p_max, per launch (algorithmic FLOPs /
-    # live launch time), and of every kernel class per cycle
-    work = perfmodel.vcycle_work(dim, W["p_max"], E, F, form=prec)
-    fl = perfmodel.residual_volume_flops(perfmodel.Shape(dim, W["p_max"], E, F))
-    achieved = fl / (vol_launch_ms * 1e-3) / 1e12
-    pk = peaks["fp64_tflops"]
-    out["roofline"] = {"bound": "alu", "kernel": f"k_volume<{dim},{W['p_max']}> (DG residual, volume + face projection)",
-                       "achieved": achieved, "peak": pk, "unit": "TFLOP/s", "frac": achieved / pk,
-                       "traffic": VOLUME_P4_TRAFFIC.get(W["name"]),
-                       "peak_source": peaks["fp64_source"], "probe_tflops": peaks["fp64_probe_tflops"],
-                       "algorithmic_flops_per_launch": fl, "ms_per_launch": vol_launch_ms,
-                       "note": "FMA-only flop model (perfmodel.residual_volume_flops)"}
-    out["rooflines"] = kernel_rooflines(prof_cycle, work, peaks, hbm_gbs, prec)
+    # roofline of the residual's largest kernel, k_volume at p_max, per launch (the operations of its
+    # formulation / live launch time), and of every kernel class per cycle
+    top = perfmodel.kernel_work(dim, W["p_max"], E, F, form=prec)
+    below = perfmodel.kernel_work(dim, W["p_max"] - 1, E, F, form=prec) if W["p_max"] > 0 else None
+    launches_top = 2 if below is None else 1 + 2 * 4   # residuals of that level in a cycle
+    ops = {u: (n - (below["residual_volume"][u] if below else 0.0)) / launches_top
+           for u, n in top["residual_volume"].items()}
+    out["roofline"] = dict(unit_roofline(ops, vol_launch_ms * 1e-3, peaks, hbm_gbs),
+                           kernel=f"k_volume<{dim},{W['p_max']}> (DG residual, volume + face projection)",
+                           traffic=VOLUME_P4_TRAFFIC.get(W["name"]),
+                           peak_source=peaks["fp64_source"], probe_tflops=peaks["fp64_probe_tflops"],
+                           operations_per_launch=ops, ms_per_launch=vol_launch_ms,
+                           note="unit that needs longest for the kernel's own operations (perfmodel.kernel_work)")
+    out["rooflines"] = unit_rooflines(prof_cycle, top, peaks, hbm_gbs)
     s.close()
     return out
 

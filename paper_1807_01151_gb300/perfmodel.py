@@ -1,8 +1,9 @@
 """Algorithmic work model of the eMG kernels (FLOPs and bytes per launch).
 
-Counts what each step of the method must compute in the formulation the kernels use,
-independent of how a kernel schedules it.  Used to turn measured kernel times into a
-roofline fraction.  Shapes: d dimensions, N modes, q = p + 2 Gauss points per direction,
+Counts what each step of the method must compute, independent of how a kernel schedules it, as
+float64 (float32 blocks: float32) multiply-adds over all five variables; `kernel_work` counts the
+operations of the formulation the kernels use, unit by unit, which turns measured kernel times into
+roofline fractions.  Shapes: d dimensions, N modes, q = p + 2 Gauss points per direction,
 Q = q^d volume points, QF = q^(d-1) points per face, 2d faces per element, B = 5N.
 """
 from dataclasses import dataclass
@@ -129,3 +130,61 @@ def vcycle_work(dim, p_max, E, F, rk_stages=4, pre_smooth=2, krylov_m=30, form=0
     w["arnoldi"][0] = krylov_m * E * (1 + nf) * 25 * FMA + sum(4 * (j + 1) * K0 * FMA for j in range(krylov_m))
     w["arnoldi"][1] = krylov_m * spmv_b + orth_b
     return w
+
+
+# ---- the kernels' own formulation ------------------------------------------------------------------
+# 32 x 32 -> 64 bit integer multiply-adds per second of the chip (independent chains in registers: 51
+# to 52 per clock and SM), and float64 operations of a point (a fused multiply-add is one).
+INT_MAD_TOPS = 16.3
+ROE_OPS = {2: 119, 3: 136}       # the Roe flux between two traces
+POINT_OPS = {2: 24, 3: 34}       # a volume point: conversions of U, pressure, fluxes
+
+
+def kernel_work(dim, p_max, E, F, rk_stages=4, pre_smooth=2, krylov_m=30, form=0):
+    """Per V-cycle and kernel class, the operations that the kernels' formulation needs of each unit:
+    int (integer multiply-adds: three to a term of a fixed-point sum), f64 and f32 (operations, a
+    multiply-add being one), bytes.  2-D is plane flow: four variables, 17 pairs of them, blocks of
+    4 N + N."""
+    nv, pairs = (4, 17) if dim == 2 else (5, 25)
+    w = {k: {"int": 0.0, "f64": 0.0, "f32": 0.0, "bytes": 0.0}
+         for k in ("residual_face_flux", "residual_volume", "diag_block_assembly", "block_lu", "prk_stage_solve",
+                   "arnoldi")}
+
+    def add(k, times, **ops):
+        for unit, n in ops.items():
+            w[k][unit] += times * n
+
+    for p in range(p_max, -1, -1):
+        s = Shape(dim, p, E, F)
+        N, Q, QF, NF, B = s.N, s.Q, s.QF, s.NF, s.B
+        fx = 3.0 if p > 0 else 0.0          # p = 0 has float64 tables and no volume term
+        n_res = 2 if p == 0 else 1 + pre_smooth * rk_stages
+        tab = E * NF * QF * N * 8           # the elements' sides of the face tables
+        add("residual_face_flux", n_res, int=fx * E * NF * QF * nv * N, f64=F * QF * ROE_OPS[dim] + E * NF * QF * nv * 2,
+            bytes=tab + E * B * 8 + F * QF * (10 + 4 + 5) * 8)
+        add("residual_volume", n_res, int=fx * E * nv * N * (Q + dim * Q + NF * QF),
+            f64=E * ((Q * POINT_OPS[dim] if p > 0 else NF * QF * nv) + 4 * nv * N),
+            bytes=tab + (E * Q * N * (1 + dim) * 8 if p > 0 else 0) + F * QF * 5 * 8 + 2 * E * B * 8)
+        if p == 0:
+            continue
+        macs = pairs * N * (Q * (dim + N) + NF * QF * (1 + N))
+        solve = (4 * N) ** 3 + N ** 3 if dim == 2 else B ** 3
+        used = (4 * N) ** 2 if dim == 2 else B * B      # entries a stage applies
+        if form == 0:
+            add("diag_block_assembly", pre_smooth, int=3.0 * E * macs, bytes=E * B * B * 8)
+            add("block_lu", pre_smooth, f64=E * solve / 3.0, bytes=2 * E * B * B * 8)
+            add("prk_stage_solve", pre_smooth * rk_stages, f64=E * used, bytes=E * (used * 8 + 3 * B * 8 + B * 4))
+        else:
+            stored = 17 * N * N if dim == 2 else B * B
+            add("diag_block_assembly", pre_smooth, f32=E * macs, bytes=E * stored * 4)
+            add("block_lu", pre_smooth, f32=E * solve, bytes=2 * E * stored * 4)
+            add("prk_stage_solve", pre_smooth * rk_stages, f32=E * used, bytes=E * (used * 4 + 3 * B * 8))
+    old = vcycle_work(dim, 0, E, F, rk_stages, pre_smooth, krylov_m, form)["arnoldi"]
+    add("arnoldi", 1, f64=old[0] / FMA, bytes=old[1])
+    return w
+
+
+def unit_times(ops, peaks, hbm_gbs):
+    """Seconds that each unit needs at its peak; peaks: fp64_tflops, fp32_tflops (two flops an operation)."""
+    return {"int": ops["int"] / (INT_MAD_TOPS * 1e12), "f64": ops["f64"] * FMA / (peaks["fp64_tflops"] * 1e12),
+            "f32": ops["f32"] * FMA / (peaks["fp32_tflops"] * 1e12), "hbm": ops["bytes"] / (hbm_gbs * 1e9)}
