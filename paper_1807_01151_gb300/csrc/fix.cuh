@@ -138,19 +138,12 @@ using FaceTab = RowTab<Lv<D, P>::N, Lv<D, P>::QF, (Lv<D, P>::QF * Lv<D, P>::N) %
 template <int D, int P>
 using GradTab = RowTab<Lv<D, P>::N, D * Lv<D, P>::Q, (D * Lv<D, P>::Q * Lv<D, P>::N) % 2 == 0>;
 
-// Ask L2 for `bytes` bytes from p (any alignment): one instruction, no register, nothing waits.
-__device__ __forceinline__ void l2_prefetch(const void* p, size_t bytes) {
-    const uint64_t a = reinterpret_cast<uint64_t>(p) & ~(uint64_t)15;
-    const unsigned n = (unsigned)((reinterpret_cast<uint64_t>(p) + bytes + 15 - a) & ~(uint64_t)15);
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(reinterpret_cast<void*>(a))), "r"(n)
-                 : "memory");
-}
-
 // Reciprocal and reciprocal square root of a float64: one third-order step (Householder's method
 // for 1/y - a and 1/y^2 - a) on the hardware's approximation, whose error of about 2^-20 becomes
 // its cube, below the rounding of the result (within 2 ulp of the exact value).  3 and 5 float64
 // operations, where the correctly rounded division and square root take the pipe for 5 and 9.  For
-// normal positive arguments; 0, denormals and infinities give an infinity or NaN.
+// normal arguments whose result is normal (the reciprocal's of either sign; a negative one's root is
+// NaN); 0, denormals and infinities give an infinity or NaN.
 __device__ __forceinline__ double rcp_h3(double a) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));

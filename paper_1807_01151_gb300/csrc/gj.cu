@@ -32,9 +32,9 @@ emg_status launch_gj_tc(emg_ctx* c, int B, float* blk, bool* built);
 // search by warp reductions, the pivot row by shuffles: no block barrier inside) and
 // publishes F and the pivot rows; (C) every warp gathers the pivot rows' entries of its own
 // columns in a warp-private buffer (no block barrier) and applies the rank-NB update,
-// s = 0 .. NB-1 in order, one FMA per term.  Pivot choice and tie rule are those of the
-// unblocked forms in gj_tile.cu and gj_cols.cu (largest |a_rk| among the unused rows, lowest
-// row on ties, the lowest unused row if no candidate is a number).  The summation order
+// s = 0 .. NB-1 in order, one FMA per term.  The pivot is the lowest of the unused rows whose |a_rk| is within
+// 2^-15 of the largest, a NaN before any number (piv_pack; the unblocked forms in gj_tile.cu and
+// gj_cols.cu take the largest itself, a NaN last).  The summation order
 // differs from the unblocked forms (results agree to float rounding, not bitwise); the
 // variants with different W compute identically.  The inverse is written column-major, as
 // by the other forms.
@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(32 * W, GjSplit<N, W>::MINB) k_gj_split(
 // times (0 = fully, only for B <= 100); 4..8 are the column-owner form with kGjWarps[v - 4]
 // warps per element (valid while a thread's share of the block stays at most 128 values);
 // 9..13 the rotating column-owner form with kGjWarps[v - 9] warps.  Blocked (14..17):
-// k_gj_blk with kGjBlkWarps[v - 14] warps (valid while a thread holds at most 64 values).  The split form
-// of 2-D levels is a family of its own.
+// k_gj_blk with kGjBlkWarps[v - 14] warps (valid while a thread holds at most 64 values, 128 with one warp).
+// The split form of 2-D levels is a family of its own, timed on whole or on packed blocks.
 // Within a family the variants do the same arithmetic in the same order, so the tuner's choice
 // never changes a result; the tuner times one family only (the blocked one where it is valid,
 // unless emg_params.block_kernels asks for the unblocked forms).

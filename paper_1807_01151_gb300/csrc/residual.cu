@@ -11,10 +11,11 @@
 // products on the integer pipe (fix.cuh); the point fluxes are float64.  With every contraction on
 // the float64 pipe (2 multiply-adds per clock and SM) the residual was at that pipe's limit: one
 // evaluation alone took 284 us on a 128 x 64 O-grid at p = 4 and 1.82 ms on 3234 hexes at p = 4, now
-// 150 us and 0.69 ms.  What bounds the parts now (128 x 64, p = 4, ncu): k_traces 20 us, the latency
-// of its staging; k_face_flux 31 us, 80 % of the float64 pipe (Roe fluxes); k_volume 74 us, issue
-// (about 5600 instructions per warp of 2 elements at 16 warps per SM, a third of them multiply-adds)
-// and 140 MB of tables.  More resident warps with fewer registers (64 to 96 a thread), other block
+// 124 us and 0.65 ms one after the other.  What bounds the parts (128 x 64, p = 4, ncu): k_traces 21 us, the latency
+// of its staging; k_face_flux 31 us, 80 % of the float64 pipe (Roe fluxes); k_volume 72 us, latency and
+// issue at 16 warps per SM (about 6700 instructions per warp of 2 elements, 34 % of the issue slots) and
+// 130 MB of tables (a quarter of the DRAM's rate).  3234 hexes, p = 4: 86, 95 (86 % of the float64 pipe) and
+// 466 us.  More resident warps with fewer registers (64 to 96 a thread), other block
 // sizes and L2 prefetches of the tables measured equal or slower.
 // ROT: a frame rotating with angular velocity omega (Eq. euler): the fluxes carry the velocity
 // relative to the frame v_r = omega x x (tabulated at the points), F_k - (v_r)_k U, the face

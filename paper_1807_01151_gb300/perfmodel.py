@@ -179,8 +179,10 @@ def kernel_work(dim, p_max, E, F, rk_stages=4, pre_smooth=2, krylov_m=30, form=0
             add("diag_block_assembly", pre_smooth, f32=E * macs, bytes=E * stored * 4)
             add("block_lu", pre_smooth, f32=E * solve, bytes=2 * E * stored * 4)
             add("prk_stage_solve", pre_smooth * rk_stages, f32=E * used, bytes=E * (used * 4 + 3 * B * 8))
-    old = vcycle_work(dim, 0, E, F, rk_stages, pre_smooth, krylov_m, form)["arnoldi"]
-    add("arnoldi", 1, f64=old[0] / FMA, bytes=old[1])
+    # the mixed forms' Krylov process is float32; the basis stays in registers
+    K0, nf = 5 * E, 2 * dim
+    macs = krylov_m * E * (1 + nf) * 25 + sum(4 * (j + 1) * K0 for j in range(krylov_m))
+    add("arnoldi", 1, bytes=krylov_m * (E * (1 + nf) * 25 * 8 + 2 * K0 * 8), **{"f32" if form else "f64": macs})
     return w
 
 
