@@ -45,7 +45,8 @@ struct DiagFx {
     // 2-D: the face points have places of their own, so that both parts run without a barrier between
     static constexpr int O_FS = TAB, O_FJ = O_FS + FP * NP;
     static constexpr int ALL = D == 2 ? O_FJ + FP * 25 : TAB;
-    // resident blocks asked of the register allocator (80 registers a thread in 2-D; 3-D p = 3: 128)
+    // resident blocks asked of the register allocator (80 registers a thread for N = 10 and 15 in 2-D, 60 and 67
+    // below; 3-D p = 1, 2, 3: 96, 103, 128)
     static constexpr int MINB = D == 2 ? (N == 15 ? 3 : N == 10 ? 4 : 5) : N == 20 ? 1 : N == 10 ? 2 : 4;
     static constexpr int SLAB = N * B;
     static constexpr int O_ACC = ALL > SLAB ? ALL : SLAB;              // 3-D: [3][N][LIVE N] words of the 96-bit sums

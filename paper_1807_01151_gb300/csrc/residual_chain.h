@@ -20,10 +20,10 @@ constexpr int volume_elems(int dim, int p) {
 // 181 x 80 p = 3 132 / 126, 150 x 70 p = 4 154 / 152 and 128 x 64 p = 4 123 / 125, but with three solvers in
 // turn 113 / 109 and 87.2 / 84.5.  3-D gains nothing at any large size with three.
 // The lines: 12000 face points (chained 0.77 to 0.96 below; 64 x 32 p = 1, 12384 of them, 1.00, with
-// three 1.16), 20000 at p = 0 (96 x 48, 18528: 0.76; 128 x 64, 33024: 1.06); 2-D, 1.6 waves of k_volume's
-// blocks (8 of its 64 threads a multiprocessor).
+// three 1.16), at p = 0 28000 in 2-D (110 x 55, 24420: 0.78; 128 x 64, 33024: 1.06) and 100000 in 3-D (7200 hexes,
+// 88800: 0.88); 2-D, 1.6 waves of k_volume's blocks (8 of its 64 threads a multiprocessor).
 inline bool residual_chains(int dim, int p, int64_t elems, int64_t face_points) {
-    if (face_points <= (p == 0 ? 20000 : 12000)) return true;
+    if (face_points <= (p > 0 ? 12000 : dim == 2 ? 28000 : 100000)) return true;
     return dim == 2 && p > 0 && 5 * (elems / volume_elems(dim, p)) >= 8 * (8 * 152);
 }
 

@@ -29,7 +29,7 @@ def chains(tmp_path_factory):
     return rule
 
 
-@pytest.mark.parametrize("case", [(2, 32, 16, 0), (2, 96, 48, 0), (2, 32, 16, 1), (2, 32, 16, 2), (2, 24, 10, 3),
+@pytest.mark.parametrize("case", [(2, 32, 16, 0), (2, 110, 55, 0), (3, 10, 12, 0), (2, 32, 16, 1), (2, 32, 16, 2), (2, 24, 10, 3),
                                   (2, 45, 21, 4), (3, 3, 4, 1), (2, 181, 80, 3), (2, 150, 70, 4), (2, 256, 128, 2)])
 def test_chained_where_it_was_measured_faster(chains, case):
     assert chains(*case)
