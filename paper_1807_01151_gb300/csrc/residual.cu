@@ -380,11 +380,11 @@ struct VolCfg {
     static constexpr int FC1 = FC0 < FIX_TERMS / L::QF ? FC0 : FIX_TERMS / L::QF;
     static constexpr int FC = FC1 < 1 ? 1 : (FC1 > L::NF ? L::NF : FC1);
     // the directions' sums are added with SH bits less: D QC 2^(56 - SH) < 2^63
-    static constexpr int SH = D * QC > 252 ? 2 : D * QC > 120 ? 1 : 0;
+    static constexpr int SH = D * QC > 120 ? 1 : 0;
     static constexpr int ROWS = QC * D > FC * L::QF ? QC * D : FC * L::QF;
     // 128 registers a thread; the quarter rows of 2-D p = 3, which fit fewer, ten blocks (50 x 25: 41.4 -> 35.8 us)
     static constexpr int MINB = S && D == 2 && P == 3 ? 10 : 512 / THREADS;
-    static_assert(QC >= 2 && FC * L::QF <= FIX_TERMS && QC <= FIX_TERMS && D * QC <= 504 && L::N <= FIX_TERMS, "exact sums");
+    static_assert(QC >= 2 && FC * L::QF <= FIX_TERMS && QC <= FIX_TERMS && D * QC <= 252 && L::N <= FIX_TERMS, "exact sums");
 };
 
 // Largest of the keys that the warp's lanes hold for their elements, one atomic per element and key.
